@@ -7,6 +7,7 @@
 // the single parameter inferred from the data) on scalars read back from the device.
 #include "mpr.h"
 #include "mpr_internal.h"
+#include "mpr_resident.h"
 
 #include <cuda_runtime.h>
 
@@ -133,6 +134,14 @@ struct mpr_ctx {
     int nsplit = 0;                      // plain passes of the tile kernel: last tiles split in two
     int late = 0;                        // plain passes of the tile kernel, 16-bit spins: own rows
                                          // loaded at their update (the state fits the L2)
+    // resident sweeps (small and middle-sized lattices, see mpr_resident.cuh)
+    resident::Plan rplan{};
+    unsigned long long* halo = nullptr;  // boundary rows in flight between blocks
+    size_t halo_bytes = 0;
+    uint32_t epoch = 0;                  // tag of the last resident pass
+    float* er = nullptr;                 // row sums of measured sweeps
+    void* rpart = nullptr;               // their tile partials
+    size_t er_bytes = 0, rpart_bytes = 0;
     // bounded Metropolis proposals (mpr_set_proposal): the half-width lives on the device in
     // scal[14], the acceptance counter of the adaptation in scal[13]
     bool prop_on = false;
@@ -241,6 +250,9 @@ void free_all(mpr_ctx* h)
     dfree(h, &h->scal, 16 * 8);
     dfree(h, &h->eseries, (size_t)h->eseries_cap * 8);
     dfree(h, &h->tmpN, (size_t)h->N * 8);
+    dfree(h, &h->halo, h->halo_bytes);
+    dfree(h, &h->er, h->er_bytes);
+    dfree(h, &h->rpart, h->rpart_bytes);
     if (h->host) cudaFreeHost(h->host);
     h->host = nullptr;
     if (h->ev0) cudaEventDestroy(h->ev0);
@@ -334,6 +346,7 @@ mpr_status init_state(mpr_ctx* h)
     // the staging (8192^2: 134 MB, where the late loads measured 1.6 % slower).
     h->late = (p.func != 0 && (p.store == kF16 || p.store == kBF16) &&
                2 * ang_bytes(h) <= ((size_t)48 << 20)) ? 1 : 0;
+    h->rplan = p.func == 1 ? resident::plan(h->L, p.store, h->nsm) : resident::Plan{};
     // TMA maps for the FP32-function kernel (false: the lattice is too narrow for its boxes)
     h->tma = TmaMaps{};
     if (p.func == 1) make_sweep_maps(h->L, p.store, h->ang, h->mb, &h->tma);
@@ -472,6 +485,90 @@ mpr_status fold_partials(mpr_ctx* h)
     return MPR_OK;
 }
 
+// A scratch array of at least `bytes`.
+template <typename T>
+mpr_status ensure_scratch(mpr_ctx* h, T** p, size_t* have, size_t bytes)
+{
+    if (bytes <= *have) return MPR_OK;
+    dfree(h, p, *have);
+    *have = 0;
+    CHECK(dalloc(h, p, bytes));
+    *have = bytes;
+    return MPR_OK;
+}
+
+// n sweeps by the resident kernel, as few launches as the scratch of measured sweeps allows.
+// *ran = false when the device cannot hold the launch's blocks at once: nothing has changed then,
+// and the handle's later sweeps run one launch per pass.
+mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
+{
+    constexpr size_t kErBytes = 16u << 20;   // row sums of the measured sweeps of one launch
+    const resident::Plan& p = h->rplan;
+    const bool measure = (flags & kMeasure) != 0;
+    *ran = true;
+    if (!p.cluster && !h->halo) {
+        CHECK(ensure_scratch(h, &h->halo, &h->halo_bytes, resident::halo_bytes(p)));
+        CU(cudaMemsetAsync(h->halo, 0, h->halo_bytes, h->stream));
+    }
+    int most = n;
+    if (measure) {
+        const size_t row = (size_t)h->L.Ly * p.G * 4, nt = (size_t)sweep_f32_blocks(h->L) * 8;
+        most = (int)std::min<size_t>((size_t)n, std::max<size_t>(1, kErBytes / row));
+        CHECK(ensure_scratch(h, &h->er, &h->er_bytes, row * (size_t)most));
+        CHECK(ensure_scratch(h, &h->rpart, &h->rpart_bytes, nt * (size_t)most));
+    }
+    resident::Args a{};
+    a.Lx = h->L.Lx;
+    a.Ly = h->L.Ly;
+    a.Lxh = h->L.Lxh;
+    a.pitch = h->L.pitch;
+    a.mpitch = h->L.mpitch;
+    a.G = p.G;
+    a.rows = p.rows;
+    for (int c = 0; c < 2; ++c) {
+        a.ang[c] = h->ang[c];
+        a.mb[c] = h->mb[c];
+        a.acc[c] = h->acc[c];
+        a.acc_hi[c] = h->acc_hi[c];
+        a.acc_lo[c] = h->acc_lo[c];
+    }
+    a.er = h->er;
+    a.halo = h->halo;
+    a.seed_lo = (uint32_t)h->opt.seed;
+    a.seed_hi = (uint32_t)(h->opt.seed >> 32);
+    a.qf = (float)h->opt.q;
+    a.nl2eTf = -1.4426950408889634f * (float)(1.0 / T);
+    a.keys = philox_sched(0u, 0u, kTagMetropolis, 0u, a.seed_lo, a.seed_hi);
+    a.err = dev_err(h);
+    a.wait_ns = 2000000000LL;
+    // FP64 sums take each sample directly (with FP16 spins too: every add is exact, so the sums are
+    // the bits of the fixed-point partials')
+    const int sample = (flags & kSample) ? (h->prec.acc == 0 ? 1 : 2) : 0;
+    for (int k = 0; k < n; k += most) {
+        const int m = std::min(most, n - k);
+        a.nsweeps = m;
+        a.sweep = h->sweep;
+        a.epoch = h->epoch;
+        const cudaError_t e = resident::launch(p, h->prec.store, measure, sample, a.qf == 0.5f, a,
+                                               h->stream);
+        if (e != cudaSuccess && k == 0) {
+            cudaGetLastError();
+            h->rplan.nb = 0;
+            *ran = false;
+            return MPR_OK;
+        }
+        CU(e);
+        if (measure)
+            CU(resident::launch_energies(h->L, h->prec.energy == 1, h->er, m, h->rpart,
+                                         h->eseries + k, h->stream));
+        h->epoch += 2u * (uint32_t)m;
+        h->launches += measure ? 3 : 1;
+        h->sweep += (uint32_t)m;
+        h->site_updates += (uint64_t)m * (uint64_t)h->Np;
+    }
+    return MPR_OK;
+}
+
 // n hybrid sweeps at temperature T; with kMeasure the raw bond sum of sweep k lands in
 // eseries[k]. Every launch goes to the handle's stream; nothing here synchronises, except the
 // one-time choice of the FP32 sweep kernel (sweep_kind), which waits for its timing events.
@@ -516,6 +613,19 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
     if (timed) {
         CHECK(harvest_profile(h));
         CU(cudaEventRecord(h->ev0, h->stream));
+    }
+    if (h->rplan.nb > 0 && h->sweep_force < 0 && !h->prop_on) {
+        bool ran = false;
+        CHECK(resident_sweeps(h, n, T, flags, &ran));
+        if (ran) {
+            if (flags == 0 && n >= 2 * (1 + kCalSweeps) && h->sweep_kind < 0) h->sweep_kind = 0;
+            if (timed) {
+                CU(cudaEventRecord(h->ev1, h->stream));
+                h->prof_pending = true;
+                h->prof_pending_launches = 2ull * (uint64_t)n;
+            }
+            return MPR_OK;
+        }
     }
     // one hybrid sweep (both colour passes) with kernel kind (0/1; ignored for FP64 functions)
     auto one = [&](int k, int kind) -> mpr_status {

@@ -1,0 +1,56 @@
+// mpr_resident.h -- host interface of the resident sweep kernel (mpr_resident.cuh): many hybrid
+// sweeps of a small or middle-sized lattice in one launch. Not part of the public ABI.
+#pragma once
+
+#include "mpr_internal.h"
+
+namespace mpr {
+namespace resident {
+
+// How a lattice is laid out over the blocks of the launch.
+struct Plan {
+    int nb = 0;          // blocks = bands of rows (0: the lattice does not run resident)
+    bool cluster = false;   // the blocks are one cluster; else a cooperative grid
+    bool pair = false;   // a thread's unit of work is a row pair (else one row) of four columns
+    int threads = 0;
+    int rows = 0;        // rows of the tallest band
+    int G = 0;           // groups of four half-lattice columns in a row
+    size_t smem = 0;     // dynamic shared memory of a block
+};
+
+struct Args {
+    int Lx, Ly, Lxh, pitch, mpitch, G, rows;
+    void* ang[2];
+    const uint32_t* mb[2];
+    double* acc[2];
+    float* acc_hi[2];
+    float* acc_lo[2];
+    float* er;                   // measured sweeps: FP32 sums of u_b . h_b per sweep, row and group
+    unsigned long long* halo;    // grid: boundary rows in flight, [colour][band][side][4 G]
+    uint32_t epoch;              // grid: tag of the pass before the launch's first
+    int nsweeps;
+    uint32_t seed_lo, seed_hi, sweep;
+    float qf, nl2eTf;
+    PhiloxSched keys;            // round keys (k[] only)
+    int* err;
+    long long wait_ns;           // limit of one wait for a neighbour
+};
+
+Plan plan(const Layout& L, int store, int nsm);
+// Bytes of the halo buffer of a plan (grid only).
+size_t halo_bytes(const Plan& p);
+// nsweeps hybrid sweeps; sample: 0 none, 1 FP64 sums, 2 Kahan sums (only with measure).
+cudaError_t launch(const Plan& p, int store, bool measure, int sample, bool qhalf, const Args& a,
+                   cudaStream_t st);
+// The raw bond sums of nsweeps measured sweeps from their row sums, in the summation order of the
+// tile kernel and its reduction (bit-identical energies): out[k] for sweep k. part: nsweeps x
+// tiles partials of scratch.
+cudaError_t launch_energies(const Layout& L, bool e32, const float* er, int nsweeps, void* part,
+                            double* out, cudaStream_t st);
+
+cudaError_t launch_f32(const Plan& p, bool measure, int sample, bool qhalf, const Args& a, cudaStream_t st);
+cudaError_t launch_f16(const Plan& p, bool measure, int sample, bool qhalf, const Args& a, cudaStream_t st);
+cudaError_t launch_bf16(const Plan& p, bool measure, int sample, bool qhalf, const Args& a, cudaStream_t st);
+
+}  // namespace resident
+}  // namespace mpr

@@ -374,6 +374,68 @@ __device__ __forceinline__ void carry_call1(GroupCarry& gc, const uint4& w)
     gc.p2 = low2(w.z, w.w);
 }
 
+// What a caller that keeps the whole lattice in shared memory (mpr_resident.cuh) hands to and takes
+// from update_row, which then neither draws random words nor stores anything: the words of the
+// row's group (calls 0, 1, 2; the second row reads its carry from gc), the old unit vectors of its
+// own four sites (their sines and cosines need not be computed again), and the results.
+struct RowIO {
+    static constexpr bool kOn = true;
+    uint4 wl0, wl1, w2;
+    float4 oc, os;        // in: (cos, sin) of q times the old angles
+    float nc[4], ns[4];   // out: of q times the new ones
+    float fsamp[4];       // out: the row's sampled angles (0: frozen)
+    float er;             // out (MEASURE): the row's sum of u_b . h_b
+};
+struct NoRowIO {
+    static constexpr bool kOn = false;
+};
+
+// Adds a row's four sampled angles to its sums by one vector read and write (the thread's columns
+// are 4-aligned, rows 128-aligned); frozen sites add 0.
+template <int SAMPLE>
+__device__ __forceinline__ void sample_row(const SweepArgs& a, size_t idx, const float* fsamp)
+{
+    if constexpr (SAMPLE == 1) {
+        double2* p = reinterpret_cast<double2*>(a.acc + idx);
+        double2 s0 = p[0], s1 = p[1];
+        s0.x += (double)fsamp[0];
+        s0.y += (double)fsamp[1];
+        s1.x += (double)fsamp[2];
+        s1.y += (double)fsamp[3];
+        p[0] = s0;
+        p[1] = s1;
+    } else if constexpr (SAMPLE == 2) {
+        // Kahan: hi carries the sum, lo the (negated) lost low-order part
+        float4* ph = reinterpret_cast<float4*>(a.acc_hi + idx);
+        float4* pl = reinterpret_cast<float4*>(a.acc_lo + idx);
+        const float4 h4 = *ph, l4 = *pl;
+        const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+        float nh[4], nl[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float yv = fsamp[k] - lv[k];
+            const float tt = hv[k] + yv;
+            nl[k] = (tt - hv[k]) - yv;
+            nh[k] = tt;
+        }
+        *ph = make_float4(nh[0], nh[1], nh[2], nh[3]);
+        *pl = make_float4(nl[0], nl[1], nl[2], nl[3]);
+    } else if constexpr (SAMPLE == 3) {
+        // FP16 spins, FP64 sums: f is an FP16 value, an integer multiple of 2^-24 below 2^3, so
+        // f * 2^24 converts to an int exactly and 16 of them fit an int32; the handle folds the
+        // partial into the FP64 sum, where every add is exact (the sum stays a multiple of 2^-24
+        // below 2^29): the same bits as adding f itself, with a 4-byte read and write per sample
+        // instead of 8-byte ones
+        int4* p = reinterpret_cast<int4*>(a.part32 + idx);
+        int4 v = *p;
+        v.x += __float2int_rn(fsamp[0] * 16777216.0f);
+        v.y += __float2int_rn(fsamp[1] * 16777216.0f);
+        v.z += __float2int_rn(fsamp[2] * 16777216.0f);
+        v.w += __float2int_rn(fsamp[3] * 16777216.0f);
+        *p = v;
+    }
+}
+
 // Metropolis + over-relaxation of the thread's four columns jb .. jb+3 of tile row ly (lattice
 // row y < Ly) of colour a.colour, reading the staged neighbours in sm; pk holds the four stored
 // values (updated in place and written back as one vector), bits their frozen bits. SAMPLE: 0
@@ -386,12 +448,13 @@ __device__ __forceinline__ void carry_call1(GroupCarry& gc, const uint4& w)
 // QM: 0 any q; 1 the caller knows q <= 1/2, so the reflected angle needs one 2 pi wrap, not two;
 // 2 q = 1/2 (the paper's value) at compile time: q*phi of the accepted angle is the proposal's
 // or the old angle's product (both computed for the energy), and r/q is r + r (exact).
-template <typename S, int R, bool MEASURE, int SAMPLE, bool SCHED, int OPAR, bool PROP, int QM,
-          int TJ, int ROW, bool HM>
+// SM: the staged neighbours (a TileSmem, or anything with rows cs[r][col], sn[r][col]); IO: RowIO or
+// NoRowIO.
+template <typename S, bool MEASURE, int SAMPLE, bool SCHED, int OPAR, bool PROP, int QM, int ROW,
+          bool HM, typename SM, typename IO>
 __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, int jb, int lj,
-                                           Pack4<S>& pk, uint32_t bits, const TileSmem<R, TJ>& sm,
-                                           double& e_d, float& e_f, float pw, int& n_acc,
-                                           GroupCarry& gc)
+                                           Pack4<S>& pk, uint32_t bits, const SM& sm, double& e_d,
+                                           float& e_f, float pw, int& n_acc, GroupCarry& gc, IO& io)
 {
     const int c = a.colour;
     S* __restrict__ own = static_cast<S*>(a.own);
@@ -448,14 +511,19 @@ __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, in
     uint4 w2 = make_uint4(0u, 0u, 0u, 0u);
     uint4 wl0 = w2, wl1 = w2;
     bool second = ROW == 1;
-    if constexpr (ROW == 2 || ROW == 0) {
+    if constexpr (IO::kOn) {
+        wl0 = io.wl0;
+        wl1 = io.wl1;
+        w2 = io.w2;
+    }
+    if constexpr (!IO::kOn && (ROW == 2 || ROW == 0)) {
         if constexpr (ROW == 2) second = ((y + c) & 1) != 0;
         wl0 = group_call<SCHED>(a, g, h, 0u);
         wl1 = group_call<SCHED>(a, g, h, 1u);
         carry_call0(gc, wl0);
         carry_call1(gc, wl1);
     }
-    if constexpr (ROW != 0) w2 = group_call<SCHED>(a, g, h, 2u);
+    if constexpr (!IO::kOn && ROW != 0) w2 = group_call<SCHED>(a, g, h, 2u);
     const uint32_t a2 = low3(gc.p2, w2.x), a3 = low3(low2(w2.y, w2.z), w2.w);
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
@@ -514,8 +582,13 @@ __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, in
             qp = mul2(splat(q), fp);
         }
         float2 s0, c0, sp, cp;
-        __sincosf(qf.x, &s0.x, &c0.x);
-        __sincosf(qf.y, &s0.y, &c0.y);
+        if constexpr (IO::kOn) {   // the same bits: computed from the stored angle when it was set
+            c0 = t == 0 ? make_float2(io.oc.x, io.oc.y) : make_float2(io.oc.z, io.oc.w);
+            s0 = t == 0 ? make_float2(io.os.x, io.os.y) : make_float2(io.os.z, io.os.w);
+        } else {
+            __sincosf(qf.x, &s0.x, &c0.x);
+            __sincosf(qf.y, &s0.y, &c0.y);
+        }
         __sincosf(qp.x, &sp.x, &cp.x);
         __sincosf(qp.y, &sp.y, &cp.y);
         // dE = E(fp) - E(f), E(phi) = -(hx cos q*phi + hy sin q*phi)
@@ -557,7 +630,7 @@ __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, in
             // site's own value converts back to its stored bits exactly
             const uint32_t packed = pack2<S>(fn.x, fn.y);
             if (t == 0) pk.v.x = packed; else pk.v.y = packed;
-            if (SAMPLE || MEASURE) {
+            if (SAMPLE || MEASURE || IO::kOn) {
                 Pack4<S> back;
                 back.v.x = packed;
                 fn = make_float2(load_as<float>(back.s[0]), load_as<float>(back.s[1]));
@@ -575,66 +648,41 @@ __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, in
         // (or padding) contributes 0 to the sums below, which leaves them unchanged
         fsamp[k0] = upd[k0] ? fn.x : 0.0f;
         fsamp[k1] = upd[k1] ? fn.y : 0.0f;
-        if (MEASURE) {
-            // every bond joins a red and a black site: sum over black sites of u_b . h_b
+        float2 sn, cs;
+        if (MEASURE || IO::kOn) {
             const float2 qn = mul2(splat(q), fn);
-            float2 sn, cs;
             __sincosf(qn.x, &sn.x, &cs.x);
             __sincosf(qn.y, &sn.y, &cs.y);
+        }
+        if constexpr (IO::kOn) {   // the new unit vectors; (0, 0) where there is no site
+            io.nc[k0] = ex[k0] ? cs.x : 0.0f;
+            io.nc[k1] = ex[k1] ? cs.y : 0.0f;
+            io.ns[k0] = ex[k0] ? sn.x : 0.0f;
+            io.ns[k1] = ex[k1] ? sn.y : 0.0f;
+        }
+        if (MEASURE) {
+            // every bond joins a red and a black site: sum over black sites of u_b . h_b
             const float2 e2 = fma2(cs, hx, mul2(sn, hy));
             ev[k0] = ex[k0] ? e2.x : 0.0f;
             ev[k1] = ex[k1] ? e2.y : 0.0f;
         }
     }
-    // Sampling: the row's four sums updated by one vector read and write (the thread's columns
-    // are 4-aligned, rows 128-aligned); frozen sites add 0.
-    if constexpr (SAMPLE == 1) {
-        double2* p = reinterpret_cast<double2*>(a.acc + idx);
-        double2 s0 = p[0], s1 = p[1];
-        s0.x += (double)fsamp[0];
-        s0.y += (double)fsamp[1];
-        s1.x += (double)fsamp[2];
-        s1.y += (double)fsamp[3];
-        p[0] = s0;
-        p[1] = s1;
-    } else if constexpr (SAMPLE == 2) {
-        // Kahan: hi carries the sum, lo the (negated) lost low-order part
-        float4* ph = reinterpret_cast<float4*>(a.acc_hi + idx);
-        float4* pl = reinterpret_cast<float4*>(a.acc_lo + idx);
-        const float4 h4 = *ph, l4 = *pl;
-        const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
-        float nh[4], nl[4];
+    if constexpr (IO::kOn) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float yv = fsamp[k] - lv[k];
-            const float tt = hv[k] + yv;
-            nl[k] = (tt - hv[k]) - yv;
-            nh[k] = tt;
-        }
-        *ph = make_float4(nh[0], nh[1], nh[2], nh[3]);
-        *pl = make_float4(nl[0], nl[1], nl[2], nl[3]);
-    } else if constexpr (SAMPLE == 3) {
-        // FP16 spins, FP64 sums: f is an FP16 value, an integer multiple of 2^-24 below 2^3, so
-        // f * 2^24 converts to an int exactly and 16 of them fit an int32; the handle folds the
-        // partial into the FP64 sum, where every add is exact (the sum stays a multiple of 2^-24
-        // below 2^29): the same bits as adding f itself, with a 4-byte read and write per sample
-        // instead of 8-byte ones
-        int4* p = reinterpret_cast<int4*>(a.part32 + idx);
-        int4 v = *p;
-        v.x += __float2int_rn(fsamp[0] * 16777216.0f);
-        v.y += __float2int_rn(fsamp[1] * 16777216.0f);
-        v.z += __float2int_rn(fsamp[2] * 16777216.0f);
-        v.w += __float2int_rn(fsamp[3] * 16777216.0f);
-        *p = v;
+        for (int k = 0; k < 4; ++k) io.fsamp[k] = fsamp[k];
+    } else {
+        sample_row<SAMPLE>(a, idx, fsamp);
     }
     if (MEASURE) {
         // the row's four FP32 terms pairwise in FP32 (two roundings of the size of the terms'
         // own), then into the thread's FP64 (or FP32) sum: one FP64 add per row instead of four,
         // on a part whose FP64 rate is a small fraction of its FP32 rate
         const float er = (ev[0] + ev[1]) + (ev[2] + ev[3]);
-        if (a.flags & kEnergyF32) e_f += er; else e_d += (double)er;
+        if constexpr (IO::kOn) io.er = er;
+        else if (a.flags & kEnergyF32) e_f += er;
+        else e_d += (double)er;
     }
-    store4(own + idx, pk);   // unchanged entries are written back with their own bits
+    if constexpr (!IO::kOn) store4(own + idx, pk);   // unchanged entries keep their own bits
 }
 
 // The tile's energy partial: warp shuffles, then the warps in order, written by thread (0, 0) to
@@ -684,16 +732,17 @@ __device__ __forceinline__ void update_row_i(int i, const SweepArgs& a, int y, i
                                              const TileSmem<R, TJ>& sm, double& e_d, float& e_f,
                                              float pw, int& n_acc, GroupCarry& gc)
 {
+    NoRowIO io;
     if constexpr (R % 2 == 0) {
         if (i & 1)
-            update_row<S, R, MEASURE, SAMPLE, SCHED, 1, PROP, QM, TJ, 1, HM>(a, y, ly, jb, lj, pk, bits,
-                                                                       sm, e_d, e_f, pw, n_acc, gc);
+            update_row<S, MEASURE, SAMPLE, SCHED, 1, PROP, QM, 1, HM>(a, y, ly, jb, lj, pk, bits, sm,
+                                                                     e_d, e_f, pw, n_acc, gc, io);
         else
-            update_row<S, R, MEASURE, SAMPLE, SCHED, 0, PROP, QM, TJ, 0, HM>(a, y, ly, jb, lj, pk, bits,
-                                                                       sm, e_d, e_f, pw, n_acc, gc);
+            update_row<S, MEASURE, SAMPLE, SCHED, 0, PROP, QM, 0, HM>(a, y, ly, jb, lj, pk, bits, sm,
+                                                                     e_d, e_f, pw, n_acc, gc, io);
     } else {
-        update_row<S, R, MEASURE, SAMPLE, SCHED, -1, PROP, QM, TJ, 2, HM>(a, y, ly, jb, lj, pk, bits, sm,
-                                                                    e_d, e_f, pw, n_acc, gc);
+        update_row<S, MEASURE, SAMPLE, SCHED, -1, PROP, QM, 2, HM>(a, y, ly, jb, lj, pk, bits, sm,
+                                                                  e_d, e_f, pw, n_acc, gc, io);
     }
 }
 
