@@ -513,7 +513,7 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
     int most = n;
     if (measure) {
         const size_t row = (size_t)h->L.Ly * p.G * 4, nt = (size_t)sweep_f32_blocks(h->L) * 8;
-        most = (int)std::min<size_t>((size_t)n, std::max<size_t>(1, kErBytes / row));
+        most = (int)std::min<size_t>((size_t)n, std::max<size_t>(3, kErBytes / row));
         CHECK(ensure_scratch(h, &h->er, &h->er_bytes, row * (size_t)most));
         CHECK(ensure_scratch(h, &h->rpart, &h->rpart_bytes, nt * (size_t)most));
     }
@@ -544,11 +544,16 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
     // FP64 sums take each sample directly (with FP16 spins too: every add is exact, so the sums are
     // the bits of the fixed-point partials')
     const int sample = (flags & kSample) ? (h->prec.acc == 0 ? 1 : 2) : 0;
-    for (int k = 0; k < n; k += most) {
-        const int m = std::min(most, n - k);
+    // a launch of the fine kernel exchanges rows at least once (its blocks write their rows back
+    // after that): two sweeps or more
+    int m = 0;
+    for (int k = 0; k < n; k += m) {
+        m = std::min(most, n - k);
+        if (n - k - m == 1) --m;
         a.nsweeps = m;
         a.sweep = h->sweep;
-        a.epoch = h->epoch;
+        a.depth = p.fine ? std::min(p.depth, 2 * (m - 1)) : 1;
+        a.epoch = p.cluster ? 0u : h->epoch;
         const cudaError_t e = resident::launch(p, h->prec.store, measure, sample, a.qf == 0.5f, a,
                                                h->stream);
         if (e != cudaSuccess && k == 0) {
@@ -561,7 +566,7 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
         if (measure)
             CU(resident::launch_energies(h->L, h->prec.energy == 1, h->er, m, h->rpart,
                                          h->eseries + k, h->stream));
-        h->epoch += 2u * (uint32_t)m;
+        h->epoch += resident::exchanges(m);
         h->launches += measure ? 3 : 1;
         h->sweep += (uint32_t)m;
         h->site_updates += (uint64_t)m * (uint64_t)h->Np;
@@ -614,7 +619,7 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
         CHECK(harvest_profile(h));
         CU(cudaEventRecord(h->ev0, h->stream));
     }
-    if (h->rplan.nb > 0 && h->sweep_force < 0 && !h->prop_on) {
+    if (h->rplan.nb > 0 && n >= 2 && h->sweep_force < 0 && !h->prop_on) {
         bool ran = false;
         CHECK(resident_sweeps(h, n, T, flags, &ran));
         if (ran) {

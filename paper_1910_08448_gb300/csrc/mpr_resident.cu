@@ -12,32 +12,50 @@ namespace {
 
 constexpr int kCluster = 16;                 // blocks of a cluster (non-portable size)
 constexpr size_t kSmem = 227 * 1024;         // shared memory of a block
-constexpr int kThreads = 640;
 
-size_t smem_of(int rows, int G, int store, bool cluster)
-{
-    const size_t P = 4 * (size_t)G + 8;
-    return (cluster ? (size_t)4 * 4 * G * 8 : 0) + 4 * (size_t)(rows + 2) * P * 4 +
-           2 * (size_t)rows * 4 * G * store_bytes(store) + 2 * (size_t)rows * G;
-}
-
-// Plan with at most `most` blocks: as few as the tallest band allows, bands of equal height but one
-// row pair.
-Plan bands(const Layout& L, int store, int most, bool cluster)
+// Bands of equal height but one row pair, at most `most` of them: as few as the tallest allows.
+Plan bands(const Layout& L, int most)
 {
     Plan p;
     const int np = (L.Ly + 1) / 2;
     const int tall = (np + most - 1) / most;
     p.nb = (np + tall - 1) / tall;
-    p.cluster = cluster;
     p.rows = 2 * tall;
     p.G = (L.Lxh + 3) / 4;
-    const int groups = tall * p.G, one_role = (groups + 31) / 32 * 32;
-    p.pair = 2 * one_role > kThreads;
-    p.threads = std::min(kThreads, p.pair ? (groups + 31) / 32 * 32 : 2 * one_role);
-    p.smem = smem_of(p.rows, p.G, store, cluster);
-    if (p.smem > kSmem) p.nb = 0;
     return p;
+}
+
+// fine_kernel with an exchange every `depth` passes; no plan where a band has fewer rows than that
+// or its units and draws more warps than a block.
+Plan fine_plan(const Layout& L, int most, bool cluster, int depth)
+{
+    Plan p = bands(L, most);
+    p.fine = true;
+    p.cluster = cluster;
+    p.depth = depth;
+    const int least = 2 * (((L.Ly + 1) / 2) / p.nb) - (L.Ly & 1);   // rows of the shortest band
+    if (p.nb > 1 && least < depth) return Plan{};
+    const int rows = p.rows + 2 * (depth - 1);
+    const size_t G = (size_t)p.G, groups = (size_t)word_groups(p.rows, depth, p.G);
+    const size_t warps = 2 * (((rows + 1) / 2 * 2 * G + 31) / 32) + (groups + 31) / 32;
+    p.threads = 32 * (int)std::min<size_t>(warps, 64);
+    p.smem = 2 * 4 * groups * 16 + (cluster ? (size_t)4 * halo_rows(depth) * 4 * G * 8 : 0) +
+             4 * (size_t)(p.rows + 2 * depth) * (4 * G + 8) * 4;
+    return p.threads <= kFineThreads && p.smem <= kSmem ? p : Plan{};
+}
+
+Plan coarse_plan(const Layout& L, int store, int most)
+{
+    Plan p = bands(L, most);
+    const size_t G = (size_t)p.G, n = (size_t)p.rows;
+    const int groups = p.rows / 2 * p.G, one_role = (groups + 31) / 32 * 32;
+    p.pair = 2 * one_role > kCoarseThreads;
+    p.threads = std::min(kCoarseThreads, p.pair ? one_role : 2 * one_role);
+    p.smem = 4 * (n + 2) * (4 * G + 8) * 4 + 2 * n * 4 * G * store_bytes(store) + 2 * n * G;
+    // a second unit per thread only in bands taller than a pair: 5000 x 60 would leave most SMs idle and
+    // take 5.7 us per pass (the tile kernel 4.1), 3500 x 600 takes 5.1 (6.0), 2300 x 1200 HDS 6.1 (9.1)
+    if ((p.pair ? groups : 2 * one_role) > kCoarseThreads && p.rows == 2) return Plan{};
+    return p.smem <= kSmem ? p : Plan{};
 }
 
 // Tile (tx, ty) of a measured black pass: the thread's rows in the tile kernel's order, its warps by
@@ -106,15 +124,28 @@ cudaError_t energies(const Layout& L, const float* er, int nsweeps, void* part, 
 Plan plan(const Layout& L, int store, int nsm)
 {
     if (store == kF64 || nsm < 1) return Plan{};
-    const long long sites = (long long)L.Lx * L.Ly;
-    if (sites <= 128 * 128) {
-        const Plan p = bands(L, store, kCluster, true);
-        if (p.nb > 0) return p;
-    }
-    return bands(L, store, nsm, false);
+    // Us per plain pass, SDS, measured. One cluster while its blocks stay short of warps: exchanges
+    // cost 0.25 us there and 0.5 us through L2, but 16 blocks hold little (64^2 0.49 against 0.82;
+    // 128^2 0.65 against 0.78; 140^2, 840 threads, 0.87 against 0.85, sampled 1.25 against 1.10).
+    // Exchanges every 4 passes while the additional rows are few (64^2: 0.49 against 0.52 every 2;
+    // 128^2 in a cluster: 0.69 against 0.65; 90 x 768 on a grid: 0.89 against 0.93), else every 2.
+    // coarse_kernel where the sites ask for more threads than a block has registers for (300 x 400
+    // fine 1.21, coarse 1.40; 512 x 400 and wider only coarse).
+    const Plan c4 = fine_plan(L, kCluster, true, 4);
+    if (c4.nb > 0 && c4.threads <= 320) return c4;
+    const Plan c2 = fine_plan(L, kCluster, true, 2);
+    if (c2.nb > 0 && c2.threads <= 448) return c2;
+    const Plan g4 = fine_plan(L, nsm, false, 4);
+    if (g4.nb > 0 && g4.threads <= 544) return g4;
+    const Plan g2 = fine_plan(L, nsm, false, 2);
+    if (g2.nb > 0) return g2;
+    return coarse_plan(L, store, nsm);
 }
 
-size_t halo_bytes(const Plan& p) { return p.cluster ? 0 : (size_t)4 * p.nb * 4 * p.G * 8; }
+size_t halo_bytes(const Plan& p)
+{
+    return p.cluster ? 0 : (size_t)4 * p.nb * halo_rows(p.depth) * 4 * p.G * 8;
+}
 
 cudaError_t launch(const Plan& p, int store, bool measure, int sample, bool qhalf, const Args& a,
                    cudaStream_t st)

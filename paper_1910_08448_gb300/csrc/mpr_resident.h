@@ -7,27 +7,32 @@
 namespace mpr {
 namespace resident {
 
+constexpr int kFineThreads = 768;
+constexpr int kCoarseThreads = 512;
+
 // How a lattice is laid out over the blocks of the launch.
 struct Plan {
     int nb = 0;          // blocks = bands of rows (0: the lattice does not run resident)
-    bool cluster = false;   // the blocks are one cluster; else a cooperative grid
-    bool pair = false;   // a thread's unit of work is a row pair (else one row) of four columns
+    bool fine = false;   // fine_kernel, else coarse_kernel
+    bool cluster = false;   // fine_kernel: the blocks are one cluster; else a cooperative grid
+    bool pair = false;   // coarse_kernel: a unit is a row pair (else one row) of four columns
     int threads = 0;
     int rows = 0;        // rows of the tallest band
+    int depth = 1;       // passes between two exchanges of boundary rows (fine_kernel: even)
     int G = 0;           // groups of four half-lattice columns in a row
     size_t smem = 0;     // dynamic shared memory of a block
 };
 
 struct Args {
-    int Lx, Ly, Lxh, pitch, mpitch, G, rows;
+    int Lx, Ly, Lxh, pitch, mpitch, G, rows, depth;
     void* ang[2];
     const uint32_t* mb[2];
     double* acc[2];
     float* acc_hi[2];
     float* acc_lo[2];
     float* er;                   // measured sweeps: FP32 sums of u_b . h_b per sweep, row and group
-    unsigned long long* halo;    // grid: boundary rows in flight, [colour][band][side][4 G]
-    uint32_t epoch;              // grid: tag of the pass before the launch's first
+    unsigned long long* halo;    // grid: boundary rows in flight, [parity][band][side][row][4 G]
+    uint32_t epoch;              // grid: tag of the last exchange before the launch
     int nsweeps;
     uint32_t seed_lo, seed_hi, sweep;
     float qf, nl2eTf;
@@ -35,6 +40,15 @@ struct Args {
     int* err;
     long long wait_ns;           // limit of one wait for a neighbour
 };
+
+// Rows per side of an exchange every K passes: K of the colour moved last, K - 2 of the other one.
+constexpr int halo_rows(int K) { return K > 1 ? 2 * K - 2 : 1; }
+
+// Philox groups (row pairs of four columns) of a pass, at most.
+constexpr int word_groups(int rows, int K, int G) { return (rows / 2 + 2 * (K / 2)) * G; }
+
+// Exchanges of a launch of nsweeps sweeps at most (the epoch grows by as many).
+constexpr uint32_t exchanges(int nsweeps) { return 2u * (uint32_t)nsweeps + 2u; }
 
 Plan plan(const Layout& L, int store, int nsm);
 // Bytes of the halo buffer of a plan (grid only).

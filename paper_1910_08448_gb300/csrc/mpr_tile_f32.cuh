@@ -374,22 +374,6 @@ __device__ __forceinline__ void carry_call1(GroupCarry& gc, const uint4& w)
     gc.p2 = low2(w.z, w.w);
 }
 
-// What a caller that keeps the whole lattice in shared memory (mpr_resident.cuh) hands to and takes
-// from update_row, which then neither draws random words nor stores anything: the words of the
-// row's group (calls 0, 1, 2; the second row reads its carry from gc), the old unit vectors of its
-// own four sites (their sines and cosines need not be computed again), and the results.
-struct RowIO {
-    static constexpr bool kOn = true;
-    uint4 wl0, wl1, w2;
-    float4 oc, os;        // in: (cos, sin) of q times the old angles
-    float nc[4], ns[4];   // out: of q times the new ones
-    float fsamp[4];       // out: the row's sampled angles (0: frozen)
-    float er;             // out (MEASURE): the row's sum of u_b . h_b
-};
-struct NoRowIO {
-    static constexpr bool kOn = false;
-};
-
 // Adds a row's four sampled angles to its sums by one vector read and write (the thread's columns
 // are 4-aligned, rows 128-aligned); frozen sites add 0.
 template <int SAMPLE>
@@ -436,6 +420,86 @@ __device__ __forceinline__ void sample_row(const SweepArgs& a, size_t idx, const
     }
 }
 
+// The moves of two same-colour sites of a row (lanes x and y): local fields hx, hy; 1 + u of the
+// proposal (op) and acceptance (oa) uniforms; stored angles f; upd0, upd1: the site is not frozen
+// (every site runs the move; a frozen one, or padding, rejects both moves, so its result is its own
+// value). Returns the angles after the moves, not yet rounded to the storage type. OLD: the caller
+// has the cosines and sines of q * f (c0, s0; the bits that __sincosf gives here). PROP, QM, HM:
+// as in update_row.
+template <int SBYTES, bool OLD, bool PROP, int QM, bool HM>
+__device__ __forceinline__ float2 move_pair(float2 hx, float2 hy, float2 op, float2 oa, float2 f,
+                                            bool upd0, bool upd1, float q, float nl2e, float width,
+                                            float inv_q, float pw, int& n_acc, float2 c0, float2 s0)
+{
+    constexpr bool QH = QM == 2;
+    const float two_pi = kTwoPiF;
+    // Metropolis: uniform proposal fp = 2 pi u (or bounded: f + pw (2u - 1), inside
+    // [0, 2 pi) only), accept if dE <= 0 or u_acc < exp(-dE/T). The first word of a site
+    // drives its proposal, the second its acceptance.
+    const float2 u_acc = add2(oa, splat(-1.0f));
+    float2 fp;
+    bool inside0 = true, inside1 = true;
+    if constexpr (PROP) {
+        const float2 u_p = add2(op, splat(-1.0f));
+        fp = fma2(splat(2.0f * pw), u_p, add2(f, splat(-pw)));
+        inside0 = (fp.x >= 0.0f) & (fp.x < two_pi);
+        inside1 = (fp.y >= 0.0f) & (fp.y < two_pi);
+    } else if constexpr (!QH) {
+        fp = fma2(splat(two_pi), op, splat(-two_pi));
+    }
+    // q * phi of the old angle and of the proposal. With q = 1/2 and uniform proposals,
+    // q * fp = pi * (1 + u) - pi rounded once, and fp = 2 * (q * fp) exactly: the same bits as
+    // fp = 2 pi (1 + u) - 2 pi rounded once, then halved.
+    const float2 qf = mul2(splat(q), f);
+    float2 qp;
+    if constexpr (QH && !PROP) {
+        qp = fma2(splat(3.14159265358979324f), op, splat(-3.14159265358979324f));
+        fp = add2(qp, qp);
+    } else {
+        qp = mul2(splat(q), fp);
+    }
+    float2 sp, cp;
+    if constexpr (!OLD) {
+        __sincosf(qf.x, &s0.x, &c0.x);
+        __sincosf(qf.y, &s0.y, &c0.y);
+    }
+    __sincosf(qp.x, &sp.x, &cp.x);
+    __sincosf(qp.y, &sp.y, &cp.y);
+    // dE = E(fp) - E(f), E(phi) = -(hx cos q*phi + hy sin q*phi)
+    const float2 dE = fma2(hx, sub2(c0, cp), mul2(hy, sub2(s0, sp)));
+    const float2 ea = make_float2(dE.x * nl2e, dE.y * nl2e);
+    // both exponentials always (no branch per site); the decisions combine without
+    // short-circuit evaluation
+    const float e0 = ex2_approx(ea.x), e1 = ex2_approx(ea.y);
+    const bool acc0 = upd0 & inside0 & ((dE.x <= 0.0f) | (u_acc.x < e0));
+    const bool acc1 = upd1 & inside1 & ((dE.y <= 0.0f) | (u_acc.y < e1));
+    if constexpr (PROP) n_acc += (acc0 ? 1 : 0) + (acc1 ? 1 : 0);
+    const float2 f1 = make_float2(acc0 ? fp.x : f.x, acc1 ? fp.y : f.y);
+    // over-relaxation: reflect q*phi about arg(h); keep it if it lands in [0, 2*pi*q].
+    // h = 0 gives NaN in atan2_doubled2, every comparison below is false and the angle
+    // stays, as the move requires.
+    float2 r;   // in [-pi - 2 pi q, pi]
+    if constexpr (QH) {
+        const float2 qf1 = make_float2(acc0 ? qp.x : qf.x, acc1 ? qp.y : qf.y);   // q * f1, exact
+        r = sub2(HM ? atan2_doubled_h2(hy, hx) : atan2_doubled2<SBYTES == 2>(hy, hx), qf1);
+    } else {
+        r = fma2(splat(-q), f1,
+                 HM ? atan2_doubled_h2(hy, hx) : atan2_doubled2<SBYTES == 2>(hy, hx));
+    }
+    // r < 0 ? r + 2 pi : r, twice: the saturated product is 1 for every negative normal r
+    // and 0 for r >= 0 and NaN; the FMA then adds 2 pi or 0 with the rounding of a plain
+    // add. (A nonzero r is never subnormal: its two terms are 0 or at least ~1e-8 in
+    // magnitude.) With q <= 1/2, r >= -2 pi and the first wrap already lands in [0, 2 pi);
+    // the second would add 0, so QM > 0 drops it without changing a bit.
+    r = fma2(splat(two_pi), make_float2(__saturatef(r.x * -0x1.0p126f),
+                                        __saturatef(r.y * -0x1.0p126f)), r);
+    if constexpr (QM == 0)
+        r = fma2(splat(two_pi), make_float2(__saturatef(r.x * -0x1.0p126f),
+                                            __saturatef(r.y * -0x1.0p126f)), r);
+    const float2 rq = QH ? add2(r, r) : mul2(r, splat(inv_q));
+    return make_float2(upd0 & (r.x <= width) ? rq.x : f1.x, upd1 & (r.y <= width) ? rq.y : f1.y);
+}
+
 // Metropolis + over-relaxation of the thread's four columns jb .. jb+3 of tile row ly (lattice
 // row y < Ly) of colour a.colour, reading the staged neighbours in sm; pk holds the four stored
 // values (updated in place and written back as one vector), bits their frozen bits. SAMPLE: 0
@@ -448,13 +512,11 @@ __device__ __forceinline__ void sample_row(const SweepArgs& a, size_t idx, const
 // QM: 0 any q; 1 the caller knows q <= 1/2, so the reflected angle needs one 2 pi wrap, not two;
 // 2 q = 1/2 (the paper's value) at compile time: q*phi of the accepted angle is the proposal's
 // or the old angle's product (both computed for the energy), and r/q is r + r (exact).
-// SM: the staged neighbours (a TileSmem, or anything with rows cs[r][col], sn[r][col]); IO: RowIO or
-// NoRowIO.
 template <typename S, bool MEASURE, int SAMPLE, bool SCHED, int OPAR, bool PROP, int QM, int ROW,
-          bool HM, typename SM, typename IO>
+          bool HM, typename SM>
 __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, int jb, int lj,
                                            Pack4<S>& pk, uint32_t bits, const SM& sm, double& e_d,
-                                           float& e_f, float pw, int& n_acc, GroupCarry& gc, IO& io)
+                                           float& e_f, float pw, int& n_acc, GroupCarry& gc)
 {
     const int c = a.colour;
     S* __restrict__ own = static_cast<S*>(a.own);
@@ -462,8 +524,7 @@ __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, in
     const float q = QH ? 0.5f : a.qf;
     // exp(-dE/T) = 2^(dE * nl2e): nl2e = -log2(e) * (1/T), the FP32 product formed by the caller
     const float nl2e = a.nl2eTf;
-    const float two_pi = kTwoPiF;
-    const float width = QH ? 3.14159265358979324f : two_pi * q;
+    const float width = QH ? 3.14159265358979324f : kTwoPiF * q;
     const float inv_q = QH ? 2.0f : 1.0f / q;
     const int o = OPAR >= 0 ? OPAR : ((y + c) & 1);
     const size_t idx = (size_t)y * a.pitch + jb;
@@ -511,19 +572,14 @@ __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, in
     uint4 w2 = make_uint4(0u, 0u, 0u, 0u);
     uint4 wl0 = w2, wl1 = w2;
     bool second = ROW == 1;
-    if constexpr (IO::kOn) {
-        wl0 = io.wl0;
-        wl1 = io.wl1;
-        w2 = io.w2;
-    }
-    if constexpr (!IO::kOn && (ROW == 2 || ROW == 0)) {
+    if constexpr (ROW == 2 || ROW == 0) {
         if constexpr (ROW == 2) second = ((y + c) & 1) != 0;
         wl0 = group_call<SCHED>(a, g, h, 0u);
         wl1 = group_call<SCHED>(a, g, h, 1u);
         carry_call0(gc, wl0);
         carry_call1(gc, wl1);
     }
-    if constexpr (!IO::kOn && ROW != 0) w2 = group_call<SCHED>(a, g, h, 2u);
+    if constexpr (ROW != 0) w2 = group_call<SCHED>(a, g, h, 2u);
     const uint32_t a2 = low3(gc.p2, w2.x), a3 = low3(low2(w2.y, w2.z), w2.w);
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
@@ -554,83 +610,14 @@ __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, in
         }
         const float2 hx = hx2[t], hy = hy2[t];
         const float2 f = make_float2(load_as<float>(pk.s[k0]), load_as<float>(pk.s[k1]));
-        // every site runs the move; a frozen site (or padding) rejects both moves, so its result
-        // is its own value
-        // Metropolis: uniform proposal fp = 2 pi u (or bounded: f + pw (2u - 1), inside
-        // [0, 2 pi) only), accept if dE <= 0 or u_acc < exp(-dE/T). The first word of a site
-        // drives its proposal, the second its acceptance.
-        const float2 u_acc = add2(oa, splat(-1.0f));
-        float2 fp;
-        bool inside0 = true, inside1 = true;
-        if constexpr (PROP) {
-            const float2 u_p = add2(op, splat(-1.0f));
-            fp = fma2(splat(2.0f * pw), u_p, add2(f, splat(-pw)));
-            inside0 = (fp.x >= 0.0f) & (fp.x < two_pi);
-            inside1 = (fp.y >= 0.0f) & (fp.y < two_pi);
-        } else if constexpr (!QH) {
-            fp = fma2(splat(two_pi), op, splat(-two_pi));
-        }
-        // q * phi of the old angle and of the proposal. With q = 1/2 and uniform proposals,
-        // q * fp = pi * (1 + u) - pi rounded once, and fp = 2 * (q * fp) exactly: the same bits as
-        // fp = 2 pi (1 + u) - 2 pi rounded once, then halved.
-        const float2 qf = mul2(splat(q), f);
-        float2 qp;
-        if constexpr (QH && !PROP) {
-            qp = fma2(splat(3.14159265358979324f), op, splat(-3.14159265358979324f));
-            fp = add2(qp, qp);
-        } else {
-            qp = mul2(splat(q), fp);
-        }
-        float2 s0, c0, sp, cp;
-        if constexpr (IO::kOn) {   // the same bits: computed from the stored angle when it was set
-            c0 = t == 0 ? make_float2(io.oc.x, io.oc.y) : make_float2(io.oc.z, io.oc.w);
-            s0 = t == 0 ? make_float2(io.os.x, io.os.y) : make_float2(io.os.z, io.os.w);
-        } else {
-            __sincosf(qf.x, &s0.x, &c0.x);
-            __sincosf(qf.y, &s0.y, &c0.y);
-        }
-        __sincosf(qp.x, &sp.x, &cp.x);
-        __sincosf(qp.y, &sp.y, &cp.y);
-        // dE = E(fp) - E(f), E(phi) = -(hx cos q*phi + hy sin q*phi)
-        const float2 dE = fma2(hx, sub2(c0, cp), mul2(hy, sub2(s0, sp)));
-        const float2 ea = make_float2(dE.x * nl2e, dE.y * nl2e);
-        // both exponentials always (no branch per site); the decisions combine without
-        // short-circuit evaluation
-        const float e0 = ex2_approx(ea.x), e1 = ex2_approx(ea.y);
-        const bool acc0 = upd[k0] & inside0 & ((dE.x <= 0.0f) | (u_acc.x < e0));
-        const bool acc1 = upd[k1] & inside1 & ((dE.y <= 0.0f) | (u_acc.y < e1));
-        if constexpr (PROP) n_acc += (acc0 ? 1 : 0) + (acc1 ? 1 : 0);
-        const float2 f1 = make_float2(acc0 ? fp.x : f.x, acc1 ? fp.y : f.y);
-        // over-relaxation: reflect q*phi about arg(h); keep it if it lands in [0, 2*pi*q].
-        // h = 0 gives NaN in atan2_doubled2, every comparison below is false and the angle
-        // stays, as the move requires.
-        float2 r;   // in [-pi - 2 pi q, pi]
-        if constexpr (QH) {
-            const float2 qf1 = make_float2(acc0 ? qp.x : qf.x, acc1 ? qp.y : qf.y);   // q * f1, exact
-            r = sub2(HM ? atan2_doubled_h2(hy, hx) : atan2_doubled2<sizeof(S) == 2>(hy, hx), qf1);
-        } else {
-            r = fma2(splat(-q), f1,
-                     HM ? atan2_doubled_h2(hy, hx) : atan2_doubled2<sizeof(S) == 2>(hy, hx));
-        }
-        // r < 0 ? r + 2 pi : r, twice: the saturated product is 1 for every negative normal r
-        // and 0 for r >= 0 and NaN; the FMA then adds 2 pi or 0 with the rounding of a plain
-        // add. (A nonzero r is never subnormal: its two terms are 0 or at least ~1e-8 in
-        // magnitude.) With q <= 1/2, r >= -2 pi and the first wrap already lands in [0, 2 pi);
-        // the second would add 0, so QM > 0 drops it without changing a bit.
-        r = fma2(splat(two_pi), make_float2(__saturatef(r.x * -0x1.0p126f),
-                                            __saturatef(r.y * -0x1.0p126f)), r);
-        if constexpr (QM == 0)
-            r = fma2(splat(two_pi), make_float2(__saturatef(r.x * -0x1.0p126f),
-                                                __saturatef(r.y * -0x1.0p126f)), r);
-        const float2 rq = QH ? add2(r, r) : mul2(r, splat(inv_q));
-        float2 fn = make_float2(upd[k0] & (r.x <= width) ? rq.x : f1.x,
-                                upd[k1] & (r.y <= width) ? rq.y : f1.y);
+        float2 fn = move_pair<sizeof(S), false, PROP, QM, HM>(hx, hy, op, oa, f, upd[k0], upd[k1], q, nl2e,
+                                                              width, inv_q, pw, n_acc, float2{}, float2{});
         if constexpr (sizeof(S) == 2) {
             // 16-bit storage: the pair's two results rounded by one paired conversion; a frozen
             // site's own value converts back to its stored bits exactly
             const uint32_t packed = pack2<S>(fn.x, fn.y);
             if (t == 0) pk.v.x = packed; else pk.v.y = packed;
-            if (SAMPLE || MEASURE || IO::kOn) {
+            if (SAMPLE || MEASURE) {
                 Pack4<S> back;
                 back.v.x = packed;
                 fn = make_float2(load_as<float>(back.s[0]), load_as<float>(back.s[1]));
@@ -648,41 +635,27 @@ __device__ __forceinline__ void update_row(const SweepArgs& a, int y, int ly, in
         // (or padding) contributes 0 to the sums below, which leaves them unchanged
         fsamp[k0] = upd[k0] ? fn.x : 0.0f;
         fsamp[k1] = upd[k1] ? fn.y : 0.0f;
-        float2 sn, cs;
-        if (MEASURE || IO::kOn) {
-            const float2 qn = mul2(splat(q), fn);
-            __sincosf(qn.x, &sn.x, &cs.x);
-            __sincosf(qn.y, &sn.y, &cs.y);
-        }
-        if constexpr (IO::kOn) {   // the new unit vectors; (0, 0) where there is no site
-            io.nc[k0] = ex[k0] ? cs.x : 0.0f;
-            io.nc[k1] = ex[k1] ? cs.y : 0.0f;
-            io.ns[k0] = ex[k0] ? sn.x : 0.0f;
-            io.ns[k1] = ex[k1] ? sn.y : 0.0f;
-        }
         if (MEASURE) {
             // every bond joins a red and a black site: sum over black sites of u_b . h_b
+            const float2 qn = mul2(splat(q), fn);
+            float2 sn, cs;
+            __sincosf(qn.x, &sn.x, &cs.x);
+            __sincosf(qn.y, &sn.y, &cs.y);
             const float2 e2 = fma2(cs, hx, mul2(sn, hy));
             ev[k0] = ex[k0] ? e2.x : 0.0f;
             ev[k1] = ex[k1] ? e2.y : 0.0f;
         }
     }
-    if constexpr (IO::kOn) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) io.fsamp[k] = fsamp[k];
-    } else {
-        sample_row<SAMPLE>(a, idx, fsamp);
-    }
+    sample_row<SAMPLE>(a, idx, fsamp);
     if (MEASURE) {
         // the row's four FP32 terms pairwise in FP32 (two roundings of the size of the terms'
         // own), then into the thread's FP64 (or FP32) sum: one FP64 add per row instead of four,
         // on a part whose FP64 rate is a small fraction of its FP32 rate
         const float er = (ev[0] + ev[1]) + (ev[2] + ev[3]);
-        if constexpr (IO::kOn) io.er = er;
-        else if (a.flags & kEnergyF32) e_f += er;
+        if (a.flags & kEnergyF32) e_f += er;
         else e_d += (double)er;
     }
-    if constexpr (!IO::kOn) store4(own + idx, pk);   // unchanged entries keep their own bits
+    store4(own + idx, pk);   // unchanged entries keep their own bits
 }
 
 // The tile's energy partial: warp shuffles, then the warps in order, written by thread (0, 0) to
@@ -732,17 +705,16 @@ __device__ __forceinline__ void update_row_i(int i, const SweepArgs& a, int y, i
                                              const TileSmem<R, TJ>& sm, double& e_d, float& e_f,
                                              float pw, int& n_acc, GroupCarry& gc)
 {
-    NoRowIO io;
     if constexpr (R % 2 == 0) {
         if (i & 1)
             update_row<S, MEASURE, SAMPLE, SCHED, 1, PROP, QM, 1, HM>(a, y, ly, jb, lj, pk, bits, sm,
-                                                                     e_d, e_f, pw, n_acc, gc, io);
+                                                                     e_d, e_f, pw, n_acc, gc);
         else
             update_row<S, MEASURE, SAMPLE, SCHED, 0, PROP, QM, 0, HM>(a, y, ly, jb, lj, pk, bits, sm,
-                                                                     e_d, e_f, pw, n_acc, gc, io);
+                                                                     e_d, e_f, pw, n_acc, gc);
     } else {
         update_row<S, MEASURE, SAMPLE, SCHED, -1, PROP, QM, 2, HM>(a, y, ly, jb, lj, pk, bits, sm,
-                                                                  e_d, e_f, pw, n_acc, gc, io);
+                                                                  e_d, e_f, pw, n_acc, gc);
     }
 }
 

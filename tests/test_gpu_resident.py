@@ -111,3 +111,17 @@ def test_two_handles_on_two_streams(mpr):
         t.join()
     for g, w in zip(got, want):
         _same(g, w)
+
+
+# One plan of each kind at its edges: a cluster that exchanges rows every 4 or 2 passes, a grid every
+# 4 or 2, or every pass with rows and with row pairs; odd heights whose last band is one row short;
+# a single band; the widest and the tallest. Runs of 2 and 3 sweeps hold the fewest exchanges.
+@pytest.mark.parametrize("Lx,Ly", [(40, 64), (64, 63), (9, 200), (112, 97), (128, 127), (60, 400), (61, 399),
+                                   (90, 767), (250, 100), (256, 255), (301, 299), (400, 300), (512, 401),
+                                   (2, 2500), (1200, 3), (1400, 1200)])
+@pytest.mark.parametrize("setup,q,acc", [("SDS", 0.5, "f64"), ("HDS", 0.8, "kahan")])
+def test_same_bits_for_every_plan(mpr, Lx, Ly, setup, q, acc):
+    pr = mpr_inputs.make_problem(Lx, Ly, 0.6, field_seed=61, mask_seed=62, periodic=True)
+    pr.mask[0, :2] = 1
+    parts = ((2, 0), (3, 2), (0, 3), (1, 1), (25, 9))
+    _same(_run(mpr, pr, setup, -1, q=q, acc=acc, parts=parts), _run(mpr, pr, setup, 0, q=q, acc=acc, parts=parts))
