@@ -94,6 +94,7 @@ struct Args {
 struct Shape {
     int cols, rpt;
 };
+constexpr int kMaxGroups = 8;   // graph mode: groups of problems, each with its own while loop
 constexpr int kShapes = 5;
 constexpr Shape kShape[kShapes] = {{128, 1}, {128, 2}, {128, 4}, {64, 1}, {64, 2}};
 constexpr int shape_rows(int s) { return 8 * (128 / kShape[s].cols) * kShape[s].rpt; }
@@ -120,13 +121,14 @@ cudaError_t batch_occupancy(int store, int shape, int* blocks_per_sm);
 // parameter of every tile kernel.
 cudaError_t batch_launch(int store, int shape, int grid, const batch::Args* args_dev,
                          const PhiloxSched& keys, cudaStream_t st, bool use_graph);
-// Graph mode: an executable graph whose device-side while loop runs red pass, black pass and the
-// finish kernel until no problem is active (or max_iters). max_tiles = blocks of a pass kernel.
+// Graph mode: an executable graph whose device-side while loop runs some sweeps (a red and a black
+// pass each) and the finish kernel until no problem is active (or max_iters): one such loop for each
+// of ng groups, side by side; group g has the arguments args_dev[g] and tiles[g] blocks in a pass.
 // qhalf: the batch's q is 1/2 (the pass kernels compiled for it, where the storage has them).
-// The black pass and the finish kernel hang on programmatic edges (each may start while its
-// predecessor's last blocks run, and waits for it before reading its results); where the
-// runtime refuses such edges, plain ones.
-cudaError_t batch_graph_build(int store, int shape, int max_tiles, bool qhalf,
+// Passes and the finish kernel hang on programmatic edges (each may start while its predecessor's
+// last blocks run, and waits for it before reading its results); where the runtime refuses such
+// edges, plain ones.
+cudaError_t batch_graph_build(int store, int shape, int ng, const int* tiles, bool qhalf,
                               const batch::Args* args_dev, const PhiloxSched& keys,
                               cudaGraphExec_t* out);
 
