@@ -131,7 +131,8 @@ struct mpr_ctx {
     int sweep_force = -1;                // mpr_set_sweep_kernel: -1 automatic, 0, 1
     long long stall_ns = 0;              // mpr_inject_tma_stall: wait limit of the next TMA pass
     int sweep_kind = -1;                 // automatic choice (-1 until made)
-    int nsplit = 0;                      // plain passes of the tile kernel: last tiles split in two
+    int nsplit = 0, nsplit_prop = 0;     // plain passes of the tile kernel: last tiles split in two
+                                         // (uniform, bounded proposals)
     int late = 0;                        // plain passes of the tile kernel, 16-bit spins: own rows
                                          // loaded at their update (the state fits the L2)
     // resident sweeps (small and middle-sized lattices, see mpr_resident.cuh)
@@ -306,6 +307,26 @@ mpr_status validate_options(const mpr_options* o)
     return MPR_OK;
 }
 
+// Plain passes of the tile kernel: how many of the T tiles (the last ones) run as two half-height tiles,
+// on S slots (resident blocks on the device).
+// - At most one wave: all of them, as the chain of a thread's rows and the uneven share of the SMs are
+//   what the pass costs (us per pass with none / all: 1500 x 2000 HDS 9.3 / 7.6, 2501 x 1333 BDS 9.5 / 8.1,
+//   2048^2 SDS 10.0 / 9.2, bounded HDS 12.0 / 10.8, 777 x 523 bounded 6.2 / 4.1). The kernels with
+//   fewer than four blocks per SM only where the halves fit one wave too (2501 x 1333 bounded SDS
+//   9.6 / 10.2, 1000 x 1700 DDS 9.0 / 9.7).
+// - Up to four waves of four blocks: the T mod S tiles of the partial one when twice as many fit a
+//   wave (4096^2 HDS 28.4 / 27.7, 2560^2 SDS 14.5 / 13.3), else half of them (3000^2 HDS 17.2 / 16.6).
+// - Beyond that the partial wave is a small share (8192^2: 1 % slower with it).
+int split_tiles(const mpr_ctx* h, bool bounded)
+{
+    const int per_sm = sweep_f32_plain_occupancy(h->prec, bounded), slots = per_sm * h->nsm;
+    const int nt = sweep_f32_blocks(h->L);
+    if (slots <= 0 || nt >= 16 * h->nsm) return 0;
+    if (nt <= slots) return per_sm >= 4 || 2 * nt <= slots ? nt : 0;
+    const int rem = nt % slots;
+    return 2 * rem <= slots ? rem : rem / 2;
+}
+
 // Allocates the precision-dependent state, maps the data, draws the initial angles and computes
 // e_s (which depends on q). Clears the chain: sweep counter, samples, temperature.
 mpr_status init_state(mpr_ctx* h)
@@ -329,18 +350,8 @@ mpr_status init_state(mpr_ctx* h)
             CU(cudaMemsetAsync(h->acc_lo[c], 0, accf_bytes(h), h->stream));
         }
     }
-    // Last wave of the tile kernel's plain passes: with T tiles and S resident blocks on the
-    // device, the last T mod S tiles would run as a partial wave; when twice that many blocks
-    // still fit one wave (and no tile column is narrow), they run as half-height tiles. Only for
-    // lattices of fewer than four waves, where the partial one is a large share of the pass
-    // (4096^2: 2048 tiles on 608 blocks, 2 % faster; at 8192^2 it measured 1 % slower).
-    h->nsplit = 0;
-    if (p.func != 0 && h->L.Lxh % 128 == 0) {
-        const int slots = sweep_f32_plain_occupancy(p) * h->nsm;
-        const int nt = sweep_f32_blocks(h->L);
-        const int rem = slots > 0 ? nt % slots : 0;
-        if (rem > 0 && 2 * rem <= slots && nt < 4 * slots) h->nsplit = rem;
-    }
+    h->nsplit = p.func != 0 ? split_tiles(h, false) : 0;
+    h->nsplit_prop = p.func == 1 ? split_tiles(h, true) : 0;
     // Own rows of a plain pass with 16-bit spins: loaded at each row's update when both colours
     // fit comfortably in the 129 MB L2 (4096^2: 33.5 MB; 1.8 % faster there), else all before
     // the staging (8192^2: 134 MB, where the late loads measured 1.6 % slower).
@@ -606,7 +617,7 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
     a.err = dev_err(h);
     a.wait_ns = 2000000000LL;   // 2 s: a TMA copy lands in microseconds
     a.stall_test = 0;
-    a.nsplit = (flags == 0) ? h->nsplit : 0;   // plain passes of the tile kernel only
+    a.nsplit = h->prop_on ? h->nsplit_prop : h->nsplit;   // read by the plain-pass launches only
     a.late = h->late;   // read by the plain-pass launches only (the red pass of a measured sweep too)
     // bounded proposals; the width adapts after every sweep that does not sample
     const bool adapt = h->prop_on && h->prop_target > 0.0 && !(flags & kSample);

@@ -94,7 +94,8 @@ int sweep_blocks(const Layout& L, const Precision& p);
 cudaError_t launch_sweep(const Precision& p, const SweepArgs& a, cudaStream_t st);
 int sweep_f32_blocks(const Layout& L);
 // Resident blocks per SM of the plain pass of the one-tile-per-block FP32 kernel.
-int sweep_f32_plain_occupancy(const Precision& p);
+int sweep_f32_plain_occupancy(const Precision& p, bool bounded);
+int sweep_f32_prop_occupancy(const Precision& p);
 cudaError_t launch_sweep_f32(const Precision& p, const SweepArgs& a, cudaStream_t st);
 cudaError_t launch_sweep_f32_prop(const Precision& p, const SweepArgs& a, cudaStream_t st);
 // FP16-function setting (func 2, FP16 spins, uniform proposals only).

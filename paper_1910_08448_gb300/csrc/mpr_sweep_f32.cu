@@ -11,28 +11,12 @@ int sweep_f32_blocks(const Layout& L)
     return ((L.Lxh + kTJ - 1) / kTJ) * ((L.Ly + tile_rows<kRows>() - 1) / tile_rows<kRows>());
 }
 
-int sweep_f32_plain_occupancy(const Precision& p)
+// Resident blocks per SM of the plain pass (the FP16-function variant has the launch bounds and shared
+// memory of the FP16-spin one).
+int sweep_f32_plain_occupancy(const Precision& p, bool bounded)
 {
-    using namespace sweep_f32_detail;
-    int n = 0;
-    cudaError_t e = cudaErrorInvalidValue;
-    switch (p.store) {
-    case kF64:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_f32_kernel<double, kRows, false, 0, false>, 256, 0);
-        break;
-    case kF32:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_f32_kernel<float, kRows, false, 0, false>, 256, 0);
-        break;
-    case kF16:
-        // (the FP16-function variant has the same launch bounds and shared memory)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_f32_kernel<__half, kRows, false, 0, false>, 256, 0);
-        break;
-    case kBF16:
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sweep_f32_kernel<__nv_bfloat16, kRows, false, 0, false>, 256, 0);
-        break;
-    default: break;
-    }
-    return e == cudaSuccess ? n : 0;
+    if (bounded) return sweep_f32_prop_occupancy(p);
+    return sweep_f32_detail::plain_occupancy<false>(p);
 }
 
 cudaError_t launch_sweep_f32(const Precision& p, const SweepArgs& a, cudaStream_t st)

@@ -28,11 +28,10 @@ constexpr int kRows = 4;      // rows per thread of the tiles (128 x 32)
 // batched kernels do: the energy partials, and so the energies, stay bit-identical between the
 // two paths.
 //
-// Last wave (plain passes, a.nsplit > 0): the grid has nsplit blocks more than tiles; the last
-// nsplit tiles run as two half-height tiles each (16 rows, blocks taken in pairs), so the final
-// partial wave of blocks has twice as many, half as long: less of the machine idles while it
-// drains. The host splits only when the half-lattice has no narrow last tile column and twice the
-// remainder still fits one wave.
+// Plain passes with a.nsplit > 0: the grid has nsplit blocks more than tiles; the last nsplit tiles run
+// as two half-height tiles each (16 rows, blocks taken in pairs): twice as many, half as long blocks
+// in the last wave, or in the only one (the host's rule gives the sizes and the times). A narrow last
+// column runs with the 64-column code there (a 32-column tile has no half).
 template <typename S, int R, bool MEASURE, int SAMPLE, bool PROP, int QM, bool HM, bool LATE>
 __device__ __forceinline__ void block_tile(const SweepArgs& a, int b, TileSmem<R>& sm, void* eslot)
 {
@@ -42,9 +41,13 @@ __device__ __forceinline__ void block_tile(const SweepArgs& a, int b, TileSmem<R
             const int nfull = (int)gridDim.x - 2 * a.nsplit;   // tiles that run whole
             if (b >= nfull) {
                 const int k = b - nfull, t = nfull + (k >> 1);
-                sweep_tile<S, R / 2, false, 0, true, true, PROP, kTJ, QM, HM, LATE>(
-                    a, t % ntx, 2 * (t / ntx) + (k & 1), *reinterpret_cast<TileSmem<R / 2>*>(&sm),
-                    eslot);
+                const int tx = t % ntx, ty = 2 * (t / ntx) + (k & 1);
+                if (tx == ntx - 1 && a.Lxh - tx * kTJ <= 64)
+                    sweep_tile<S, R / 4, false, 0, true, true, PROP, 64, QM, HM, LATE>(
+                        a, 2 * tx, ty, *reinterpret_cast<TileSmem<R / 4, 64>*>(&sm), eslot);
+                else
+                    sweep_tile<S, R / 2, false, 0, true, true, PROP, kTJ, QM, HM, LATE>(
+                        a, tx, ty, *reinterpret_cast<TileSmem<R / 2>*>(&sm), eslot);
                 return;
             }
         }
@@ -125,6 +128,29 @@ cudaError_t dispatch_mode(const Precision& p, const SweepArgs& a, cudaStream_t s
     if (sample == 0) return go<S, false, 0, PROP, HM>(a, st);
     if (sample == 1) return go<S, false, 1, PROP, HM>(a, st);
     return go<S, false, 2, PROP, HM>(a, st);
+}
+
+// (asked once: every device is the same part)
+template <typename S, bool PROP> int occupancy_of()
+{
+    static const int n = [] {
+        int v = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                   &v, sweep_f32_kernel<S, kRows, false, 0, PROP>, 256, 0) == cudaSuccess ? v : 0;
+    }();
+    return n;
+}
+
+template <bool PROP>
+int plain_occupancy(const Precision& p)
+{
+    switch (p.store) {
+    case kF64: return occupancy_of<double, PROP>();
+    case kF32: return occupancy_of<float, PROP>();
+    case kF16: return occupancy_of<__half, PROP>();
+    case kBF16: return occupancy_of<__nv_bfloat16, PROP>();
+    default: return 0;
+    }
 }
 
 template <bool PROP>

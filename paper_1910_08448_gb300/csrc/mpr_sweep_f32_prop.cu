@@ -9,4 +9,6 @@ cudaError_t launch_sweep_f32_prop(const Precision& p, const SweepArgs& a, cudaSt
     return sweep_f32_detail::launch_store<true>(p, a, st);
 }
 
+int sweep_f32_prop_occupancy(const Precision& p) { return sweep_f32_detail::plain_occupancy<true>(p); }
+
 }  // namespace mpr
