@@ -9,6 +9,8 @@
 // Templated on PROP (bounded Metropolis proposals): mpr_sweep_f32.cu instantiates the uniform
 // proposal variants, mpr_sweep_f32_prop.cu the bounded ones, so the two compile in parallel.
 #pragma once
+#include <type_traits>
+
 #include "mpr_tile_f32.cuh"
 
 namespace mpr {
@@ -64,7 +66,7 @@ __device__ __forceinline__ void block_tile(const SweepArgs& a, int b, TileSmem<R
         sweep_tile<S, R, MEASURE, SAMPLE, true, true, PROP, kTJ, QM, HM, LATE>(a, tx, ty, sm, eslot);
 }
 
-template <typename S, int R, bool MEASURE, int SAMPLE, bool PROP, bool HM = false, bool LATE = false>
+template <typename S, int R, bool MEASURE, int SAMPLE, bool PROP, int QM, bool HM = false, bool LATE = false>
 __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 2
                                        : ((PROP && (MEASURE || SAMPLE || sizeof(S) == 4)) ? 3 : 4))
     sweep_f32_kernel(const SweepArgs a)
@@ -76,22 +78,19 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 2
     void* eslot = nullptr;
     if (MEASURE)
         eslot = static_cast<char*>(a.epart) + (size_t)b * ((a.flags & kEnergyF32) ? 4 : 8);
-    // the plain pass (most passes) with 16-bit spins has a copy for q = 1/2 (the paper's value
-    // and the default) with q a compile-time constant; the branch is uniform over the grid (with
-    // FP32 spins the second copy would spill registers)
-    if constexpr (!MEASURE && SAMPLE == 0 && sizeof(S) == 2) {
+    if constexpr (QM < 0) {   // uniform over the grid
         if (a.qf == 0.5f) {
             block_tile<S, R, MEASURE, SAMPLE, PROP, 2, HM, LATE>(a, b, sm, eslot);
             return;
         }
     }
-    block_tile<S, R, MEASURE, SAMPLE, PROP, 0, HM, LATE>(a, b, sm, eslot);
+    block_tile<S, R, MEASURE, SAMPLE, PROP, QM < 0 ? 0 : QM, HM, LATE>(a, b, sm, eslot);
 }
 
 // Launched as a programmatic dependent launch: while the previous pass's last blocks finish, this
 // pass's blocks are scheduled and load their own rows (see sweep_tile).
-template <typename S, bool MEASURE, int SAMPLE, bool PROP, bool HM = false>
-cudaError_t go(const SweepArgs& a, cudaStream_t st)
+template <typename S, bool MEASURE, int SAMPLE, bool PROP, int QM, bool HM>
+cudaError_t go_q(const SweepArgs& a, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(((a.Lxh + kTJ - 1) / kTJ) * ((a.Ly + tile_rows<kRows>() - 1) / tile_rows<kRows>())
@@ -105,9 +104,29 @@ cudaError_t go(const SweepArgs& a, cudaStream_t st)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if constexpr (!MEASURE && SAMPLE == 0 && !PROP && sizeof(S) == 2) {
-        if (a.late) return cudaLaunchKernelEx(&cfg, sweep_f32_kernel<S, kRows, false, 0, false, HM, true>, a);
+        if (a.late) return cudaLaunchKernelEx(&cfg, sweep_f32_kernel<S, kRows, false, 0, false, QM, HM, true>, a);
     }
-    return cudaLaunchKernelEx(&cfg, sweep_f32_kernel<S, kRows, MEASURE, SAMPLE, PROP, HM>, a);
+    return cudaLaunchKernelEx(&cfg, sweep_f32_kernel<S, kRows, MEASURE, SAMPLE, PROP, QM, HM>, a);
+}
+
+// Where q = 1/2 (the paper's value and the default) is a compile-time constant (QM = 2):
+// - plain uniform passes with 16-bit spins: a copy beside the general one in the same kernel (-1);
+// - FP16 spins otherwise, and plain bounded passes with BF16 spins: kernels of their own (us per pass at
+//   8192^2: HDS sampled 142.2 / 138.5, HDH 113.6 / 108.7, bounded HDS 125.1 / 117.7, bounded BDS 129.4 / 125.6);
+// - the rest nowhere: they spill more registers with it (SDS 115.5 / 123.1, sampled 209 / 218; BDS sampled
+//   the same).
+template <typename S, bool MEASURE, int SAMPLE, bool PROP, bool HM = false>
+cudaError_t go(const SweepArgs& a, cudaStream_t st)
+{
+    constexpr bool plain = !MEASURE && SAMPLE == 0;
+    constexpr bool half = std::is_same<S, __half>::value;
+    if constexpr (sizeof(S) == 2 && plain && !PROP && !HM)
+        return go_q<S, MEASURE, SAMPLE, PROP, -1, HM>(a, st);
+    else if constexpr (half || (sizeof(S) == 2 && plain && PROP))
+        return a.qf == 0.5f ? go_q<S, MEASURE, SAMPLE, PROP, 2, HM>(a, st)
+                            : go_q<S, MEASURE, SAMPLE, PROP, 0, HM>(a, st);
+    else
+        return go_q<S, MEASURE, SAMPLE, PROP, 0, HM>(a, st);
 }
 
 template <typename S, bool PROP, bool HM = false>
@@ -133,10 +152,11 @@ cudaError_t dispatch_mode(const Precision& p, const SweepArgs& a, cudaStream_t s
 // (asked once: every device is the same part)
 template <typename S, bool PROP> int occupancy_of()
 {
+    constexpr int kAsked = sizeof(S) != 2 ? 0 : PROP ? 2 : -1;
     static const int n = [] {
         int v = 0;
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                   &v, sweep_f32_kernel<S, kRows, false, 0, PROP>, 256, 0) == cudaSuccess ? v : 0;
+                   &v, sweep_f32_kernel<S, kRows, false, 0, PROP, kAsked>, 256, 0) == cudaSuccess ? v : 0;
     }();
     return n;
 }
