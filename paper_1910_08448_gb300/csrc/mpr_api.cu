@@ -426,8 +426,7 @@ mpr_status create_common(int Lx, int Ly, const double* values, const unsigned ch
         return bail(fail(MPR_ERR_OOM, "pinned host allocation failed"));
     const int nmm = 256;
     {
-        const int sb = sweep_blocks(h->L, h->prec), sf = sweep_f32_blocks(h->L);
-        size_t need = (size_t)std::max(sb, sf) * 8;
+        size_t need = 0;
         size_t a = (size_t)sample_energy_blocks(h->L) * 16;
         size_t b = (size_t)energy_blocks(h->L) * 8;
         size_t c = (size_t)nmm * 32;
@@ -613,7 +612,6 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
     a.qf = (float)h->opt.q;
     a.invTf = (float)(1.0 / T);
     a.nl2eTf = -1.4426950408889634f * a.invTf;   // FP32 product, as the batched kernels form it
-    a.epart = h->part;
     a.err = dev_err(h);
     a.wait_ns = 2000000000LL;   // 2 s: a TMA copy lands in microseconds
     a.stall_test = 0;
@@ -643,9 +641,15 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
             return MPR_OK;
         }
     }
+    // measured sweeps: the energy partials of up to `most` sweeps, then one launch sums them all (one
+    // small launch after every sweep kept the next pass from starting: 4 us of each)
+    const size_t epart = (size_t)nblk * (h->prec.energy == 1 ? 4 : 8);
+    const int most = (int)std::min<size_t>((size_t)n, std::max<size_t>(1, ((size_t)4 << 20) / epart));
+    if (flags & kMeasure) CHECK(ensure_scratch(h, &h->rpart, &h->rpart_bytes, epart * (size_t)most));
     // one hybrid sweep (both colour passes) with kernel kind (0/1; ignored for FP64 functions)
     auto one = [&](int k, int kind) -> mpr_status {
         a.sweep = h->sweep;
+        if (flags & kMeasure) a.epart = static_cast<char*>(h->rpart) + (size_t)(k % most) * epart;
         for (int c = 0; c < 2; ++c) {
             a.colour = c;
             a.ph = philox_sched(a.sweep, a.problem, kTagMetropolis, (uint32_t)c, a.seed_lo, a.seed_hi);
@@ -668,9 +672,12 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
                     : kind == 1 ? launch_sweep_f32_tma(h->prec, a, h->tma, h->nsm, h->stream)
                                 : launch_sweep_f32(h->prec, a, h->stream));
         }
-        if (flags & kMeasure) CU(launch_reduce(h->prec, h->part, nblk, h->eseries + k, h->stream));
+        const bool sum = (flags & kMeasure) && (k % most == most - 1 || k + 1 == n);
+        if (sum)
+            CU(resident::launch_sums(h->rpart, nblk, k % most + 1, h->prec.energy == 1,
+                                     h->eseries + (k - k % most), h->stream));
         if (adapt) CU(launch_adapt_width(h->scal + 14, prop_count(h), h->Np, h->prop_target, h->stream));
-        h->launches += ((flags & kMeasure) ? 3 : 2) + (adapt ? 1 : 0);
+        h->launches += 2 + (sum ? 1 : 0) + (adapt ? 1 : 0);
         // int32 partials hold at most 16 samples: fold them into the FP64 sums then
         if ((flags & kSample) && h->part32[0] && ++h->pending32 == 16) CHECK(fold_partials(h));
         ++h->sweep;

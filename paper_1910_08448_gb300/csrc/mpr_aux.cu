@@ -489,15 +489,6 @@ cudaError_t launch_energy_fp64(const Layout& L, const Precision& p, const void* 
     });
 }
 
-cudaError_t launch_reduce(const Precision& p, const void* part, int n, double* out, cudaStream_t st)
-{
-    if (p.energy == 0)
-        reduce_kernel<double><<<1, kThreads, 0, st>>>(static_cast<const double*>(part), n, out);
-    else
-        reduce_kernel<float><<<1, kThreads, 0, st>>>(static_cast<const float*>(part), n, out);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_predict(const Layout& L, const Precision&, const double* z,
                            const unsigned char* mask, const double* range, const double* acc0,
                            const double* acc1, const float* hi0, const float* lo0,

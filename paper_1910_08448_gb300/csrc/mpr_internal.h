@@ -122,8 +122,6 @@ cudaError_t launch_energy_fp64(const Layout& L, const Precision& p, const void* 
                                const void* ang1, double q, double* part, int nblk, double* out,
                                cudaStream_t st);
 int energy_blocks(const Layout& L);
-cudaError_t launch_reduce(const Precision& p, const void* part, int n, double* out,
-                          cudaStream_t st);
 cudaError_t launch_predict(const Layout& L, const Precision& p, const double* z,
                            const unsigned char* mask, const double* range, const double* acc0,
                            const double* acc1, const float* hi0, const float* lo0,

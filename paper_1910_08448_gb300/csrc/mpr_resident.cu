@@ -115,8 +115,7 @@ cudaError_t energies(const Layout& L, const float* er, int nsweeps, void* part, 
     const int nt = sweep_f32_blocks(L), G = (L.Lxh + 3) / 4;
     E* p = static_cast<E*>(part);
     tile_sums_kernel<E><<<dim3(nt, nsweeps), dim3(32, 8), 0, st>>>(er, L.Ly, L.Lxh, G, nt, p);
-    sweep_sums_kernel<E><<<nsweeps, 256, 0, st>>>(p, nt, out);
-    return cudaGetLastError();
+    return launch_sums(p, nt, nsweeps, sizeof(E) == 4, out, st);
 }
 
 }  // namespace
@@ -156,6 +155,13 @@ cudaError_t launch(const Plan& p, int store, bool measure, int sample, bool qhal
     case kBF16: return launch_bf16(p, measure, sample, qhalf, a, st);
     default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_sums(const void* part, int n, int nsweeps, bool e32, double* out, cudaStream_t st)
+{
+    if (e32) sweep_sums_kernel<float><<<nsweeps, 256, 0, st>>>(static_cast<const float*>(part), n, out);
+    else sweep_sums_kernel<double><<<nsweeps, 256, 0, st>>>(static_cast<const double*>(part), n, out);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_energies(const Layout& L, bool e32, const float* er, int nsweeps, void* part,

@@ -56,6 +56,8 @@ size_t halo_bytes(const Plan& p);
 // nsweeps hybrid sweeps; sample: 0 none, 1 FP64 sums, 2 Kahan sums (only with measure).
 cudaError_t launch(const Plan& p, int store, bool measure, int sample, bool qhalf, const Args& a,
                    cudaStream_t st);
+// out[k] = the fixed-order sum of the n partials of sweep k (reduce_kernel's order), a block per sweep.
+cudaError_t launch_sums(const void* part, int n, int nsweeps, bool e32, double* out, cudaStream_t st);
 // The raw bond sums of nsweeps measured sweeps from their row sums, in the summation order of the
 // tile kernel and its reduction (bit-identical energies): out[k] for sweep k. part: nsweeps x
 // tiles partials of scratch.

@@ -48,3 +48,24 @@ def test_half_height_tiles_give_the_same_states(mpr, Lx, Ly, setup, bounded, q):
     pr = mpr_inputs.make_problem(Lx, Ly, 0.6, field_seed=21, mask_seed=22, periodic=True)
     pr.mask[0, :2] = 1
     assert np.array_equal(_state(mpr, pr, setup, bounded, 5, 0, q), _state(mpr, pr, setup, bounded, 0, 5, q))
+
+
+@pytest.mark.parametrize("setup", ["HDS", "HSS"])
+def test_energies_of_more_sweeps_than_one_sum_takes(mpr, setup):
+    """8192^2: the partials of 64 (FP32 energies: 128) measured sweeps are summed at once."""
+    pr = mpr_inputs.make_problem(8192, 8192, 0.9, field_seed=23, mask_seed=24, periodic=True)
+    n = 64 if setup == "HDS" else 128
+    means = []
+    for runs in ((n + 5,), (n - 1, 6)):
+        h = mpr.mpr_create(pr.z, pr.mask)
+        try:
+            mpr.mpr_set_options(h, setup, seed=3)
+            mpr.mpr_set_temperature(h, 0.065)
+            total = 0.0
+            for r in runs:
+                mpr.mpr_run(h, 0, r)
+                total += r * mpr.mpr_get_info(h)["e_bond_mean"]
+            means.append(total / (n + 5))
+        finally:
+            mpr.mpr_destroy(h)
+    assert abs(means[0] - means[1]) <= 1e-13 * abs(means[1])
