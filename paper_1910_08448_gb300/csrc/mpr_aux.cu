@@ -165,18 +165,33 @@ __global__ void __launch_bounds__(kThreads) sample_energy_kernel(Layout L,
     }
 }
 
-__global__ void sample_energy_final(const double* __restrict__ psum, const long long* __restrict__ pcnt,
-                                    int nblk, double* __restrict__ out)
+// One block: a thread added up a chain of 1024 partials in 86 us.
+__global__ void __launch_bounds__(kThreads) sample_energy_final(const double* __restrict__ psum,
+                                                                const long long* __restrict__ pcnt,
+                                                                int nblk, double* __restrict__ out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double ss[kThreads];
+    __shared__ long long sc[kThreads];
     double s = 0.0;
     long long n = 0;
-    for (int b = 0; b < nblk; ++b) {
+    for (int b = threadIdx.x; b < nblk; b += kThreads) {
         s += psum[b];
         n += pcnt[b];
     }
-    out[0] = n > 0 ? -s / (double)n : 0.0;
-    out[1] = (double)n;
+    ss[threadIdx.x] = s;
+    sc[threadIdx.x] = n;
+    __syncthreads();
+    for (int w = kThreads / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w) {
+            ss[threadIdx.x] += ss[threadIdx.x + w];
+            sc[threadIdx.x] += sc[threadIdx.x + w];
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        out[0] = sc[0] > 0 ? -ss[0] / (double)sc[0] : 0.0;
+        out[1] = (double)sc[0];
+    }
 }
 
 // --------------------------------------------------------------------------------------------
@@ -460,7 +475,7 @@ cudaError_t launch_sample_energy(const Layout& L, const double* z, const unsigne
                                  long long* part_cnt, int nblk, double* out2, cudaStream_t st)
 {
     sample_energy_kernel<<<nblk, kThreads, 0, st>>>(L, z, mask, range, q, part_sum, part_cnt);
-    sample_energy_final<<<1, 32, 0, st>>>(part_sum, part_cnt, nblk, out2);
+    sample_energy_final<<<1, kThreads, 0, st>>>(part_sum, part_cnt, nblk, out2);
     return cudaGetLastError();
 }
 
