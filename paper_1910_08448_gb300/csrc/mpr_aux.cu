@@ -224,35 +224,33 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
         const int j = sx * 30 + lane - 1, y0 = sy * rows;
         const int y1 = y0 + rows < L.Ly ? y0 + rows : L.Ly;
         // a red angle at column j of row y (0 where there is none)
+        auto is_red = [&](int y) { return j >= 0 && y >= 0 && y < L.Ly && 2 * j + (y & 1) < L.Lx; };
         auto red_at = [&](int y) -> V {
-            return j >= 0 && y >= 0 && y < L.Ly && 2 * j + (y & 1) < L.Lx
-                       ? load_as<V>(red[(size_t)y * L.pitch + j]) : (V)0;
+            return is_red(y) ? load_as<V>(red[(size_t)y * L.pitch + j]) : (V)0;
+        };
+        auto unit_at = [&](int y, V f) {
+            return energy::neighbour(energy::unit_of_turn(tab, fixed::turns(f, k)), is_red(y));
         };
         V fu = red_at(y0 - 1), fm = red_at(y0);
         bool oku = fixed::in_range(fu), okm = fixed::in_range(fm);
-        uint64_t tu = fixed::turns(fu, k), tm = fixed::turns(fm, k);
-        int64_t acc = 0;   // at most 4 x 16 terms of 2^50
+        energy::Vec uu = unit_at(y0 - 1, fu), um = unit_at(y0, fm);
+        int64_t acc = 0;   // at most 16 terms of 2^52
         for (int y = y0; y < y1; ++y) {
             const V fd = red_at(y + 1);
             const bool okd = fixed::in_range(fd);
-            const uint64_t td = fixed::turns(fd, k);
+            const energy::Vec ud = unit_at(y + 1, fd);
             const int o = (y + 1) & 1;   // black: x = 2j + o, red neighbours at columns j+o-1, j+o
             const int x = 2 * j + o;
             const bool has = lane >= 1 && lane <= 30 && j < L.Lxh && x < L.Lx;
             const V fb = has ? load_as<V>(black[(size_t)y * L.pitch + j]) : (V)0;
             const bool ok = okd && okm && oku && fixed::in_range(fb);
             if (__all_sync(0xffffffffu, ok)) {
-                const uint64_t tb = fixed::turns(fb, k);
-                const uint64_t ts = o ? __shfl_down_sync(0xffffffffu, tm, 1)
-                                      : __shfl_up_sync(0xffffffffu, tm, 1);
-                const uint64_t tl = o ? tm : ts, tr = o ? ts : tm;
-                const int64_t cl = energy::term(fixed::cos_turn(tab, tb - tl));
-                const int64_t cr = energy::term(fixed::cos_turn(tab, tb - tr));
-                const int64_t cu = energy::term(fixed::cos_turn(tab, tb - tu));
-                const int64_t cd = energy::term(fixed::cos_turn(tab, tb - td));
-                if (has)
-                    acc += (x > 0 ? cl : 0) + (x + 1 < L.Lx ? cr : 0) + (y > 0 ? cu : 0) +
-                           (y + 1 < L.Ly ? cd : 0);
+                const energy::Vec us =
+                    o ? energy::Vec{__shfl_down_sync(0xffffffffu, um.c, 1), __shfl_down_sync(0xffffffffu, um.s, 1)}
+                      : energy::Vec{__shfl_up_sync(0xffffffffu, um.c, 1), __shfl_up_sync(0xffffffffu, um.s, 1)};
+                const energy::Vec h{(um.c + us.c) + (uu.c + ud.c), (um.s + us.s) + (uu.s + ud.s)};
+                const int64_t e = energy::term(energy::unit_of_turn(tab, fixed::turns(fb, k)), h);
+                acc += has ? e : 0;
             } else {
                 const V fs = o ? __shfl_down_sync(0xffffffffu, fm, 1)
                                : __shfl_up_sync(0xffffffffu, fm, 1);
@@ -268,8 +266,8 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
             }
             fu = fm;
             fm = fd;
-            tu = tm;
-            tm = td;
+            uu = um;
+            um = ud;
             oku = okm;
             okm = okd;
         }

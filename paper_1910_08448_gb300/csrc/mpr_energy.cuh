@@ -1,12 +1,13 @@
 // mpr_energy.cuh -- sums of bond energies cos[q(phi_i - phi_j)] (Eq. 2) in 64-bit fixed point
 // (mpr_fixed.cuh), for the energy of a state and of the measured sample.
 //
-// What bounds them: an FP64 cosine is about 20 instructions of a unit that issues 2 per SM and
-// clock. Here an angle becomes a fraction of a turn once (about 18 integer instructions), a bond
-// is the cosine of a wrapped difference (about 55), and a warp walks down a strip of columns so
-// that each angle is loaded and converted once: the right neighbour comes by a shuffle, the row
-// above is still in a register. Each cosine is off by at most 2^-56 and is added as a 50-bit
-// fixed-point integer, so a sum does not depend on its order; FP64 enters once per strip.
+// What bounds them: integer multiplies. (An FP64 cosine is about 20 instructions of a unit that issues
+// 2 per SM and clock.) A warp walks down a strip of columns: each angle is loaded once and becomes a unit
+// vector once, a site's bonds are one product of its vector with the sum of its neighbours', which
+// come by shuffle or are still in a register from the row above: 229 us at 4096^2 (one cosine per bond,
+// of the wrapped difference of the angles, 253 us; FP64 cosines 1625 us). Each term is off by at most
+// 2^-55 and is added as a 50-bit fixed-point integer, so a sum does not depend on its order; FP64
+// enters once per strip.
 #pragma once
 
 #include "mpr_device.cuh"
@@ -29,8 +30,28 @@ inline int strip_rows(long long strips, int Ly)
     return r < 2 ? 2 : r > kMaxRows ? kMaxRows : (int)r;
 }
 
-// A bond's cosine (62 fraction bits) as a 50-bit fixed-point term, rounded to nearest.
-__device__ __forceinline__ int64_t term(int64_t c) { return (c + (1 << 11)) >> 12; }
+// A unit vector with 62 fraction bits, and with 60 as a neighbour (four of them add up below 2^63).
+struct Vec {
+    int64_t c, s;
+};
+__device__ __forceinline__ Vec unit_of_turn(const fixed::Dir* tab, uint64_t t)
+{
+    Vec v;
+    fixed::sincos_turn(tab, t, &v.c, &v.s);
+    return v;
+}
+__device__ __forceinline__ Vec neighbour(Vec v, bool there)
+{
+    return Vec{there ? (v.c + 2) >> 2 : 0, there ? (v.s + 2) >> 2 : 0};
+}
+
+// u . h (62 and 60 fraction bits) as a 50-bit fixed-point term, rounded to nearest.
+__device__ __forceinline__ int64_t term(Vec u, Vec h)
+{
+    const int64_t e = fixed::mulhi(fixed::split(u.c), fixed::split(h.c)) +
+                      fixed::mulhi(fixed::split(u.s), fixed::split(h.s));
+    return (e + (1 << 7)) >> 8;
+}
 constexpr double kTermUnit = 0x1p-50;
 
 // Signed angles below 7.5 in size; other values (and NaN) are the caller's FP64 case.

@@ -164,15 +164,6 @@ MPR_HD void sincos_turn(const Dir* tab, uint64_t t, int64_t* c, int64_t* s)
     *s = d.s + (((mulhi(S, m.cm1) >> 5) + mulhi(C, m.sn)) >> 5);
 }
 
-MPR_HD int64_t cos_turn(const Dir* tab, uint64_t t)
-{
-    const uint32_t k = (uint32_t)((t + (1ull << 53)) >> 54) & (kDirs - 1);
-    const int64_t rt = (int64_t)(t - ((uint64_t)k << 54));
-    const Dir d = tab[k];
-    const Small m = small_angle(rt);
-    return d.c + (((mulhi(split(d.c), m.cm1) >> 5) - mulhi(split(d.s), m.sn)) >> 5);
-}
-
 // ---- angles to turns ----------------------------------------------------------------------------
 
 // q / (2 pi) with 65 fraction bits: turns of q * phi per radian of phi (q <= 1).

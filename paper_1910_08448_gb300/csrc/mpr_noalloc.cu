@@ -58,27 +58,27 @@ __global__ void __launch_bounds__(kThreads) bond_partials(int Lx, int Ly, int ro
         const bool has = x < Lx, mine = lane < 31 && has, right = mine && x + 1 < Lx;
         const double* p = phi + (size_t)y0 * Lx + x;
         double f = has ? *p : 0.0, fb = 0.0;
-        uint64_t t = energy::turns_signed(f, k), tb;
+        energy::Vec u = energy::unit_of_turn(tab, energy::turns_signed(f, k)), ub;
         bool ok = energy::in_range_signed(f), okb;
-        int64_t acc = 0;   // at most 2 x 16 terms of 2^50
+        int64_t acc = 0;   // at most 16 terms of 2^51
         for (int y = y0; y < y1; ++y) {
             const bool below = y + 1 < Ly;
             p += Lx;
             fb = has && below ? *p : 0.0;
             okb = energy::in_range_signed(fb);
-            tb = energy::turns_signed(fb, k);
+            ub = energy::unit_of_turn(tab, energy::turns_signed(fb, k));
             if (__all_sync(0xffffffffu, ok && okb)) {
-                const uint64_t tr = __shfl_down_sync(0xffffffffu, t, 1);
-                const int64_t cr = energy::term(fixed::cos_turn(tab, t - tr));
-                const int64_t cd = energy::term(fixed::cos_turn(tab, t - tb));
-                acc += (right ? cr : 0) + (mine && below ? cd : 0);
+                const energy::Vec ur{__shfl_down_sync(0xffffffffu, u.c, 1), __shfl_down_sync(0xffffffffu, u.s, 1)};
+                const energy::Vec r = energy::neighbour(ur, right), d = energy::neighbour(ub, below);
+                const int64_t e = energy::term(u, energy::Vec{r.c + d.c, r.s + d.s});
+                acc += mine ? e : 0;
             } else {
                 const double fr = __shfl_down_sync(0xffffffffu, f, 1);
                 if (right) sum += cos(q * (f - fr));
                 if (mine && below) sum += cos(q * (f - fb));
             }
             f = fb;
-            t = tb;
+            u = ub;
             ok = okb;
         }
         sum += (double)acc * energy::kTermUnit;

@@ -33,7 +33,7 @@ int main()
         if (m == 's' && scanf("%llu", &t) == 1) {
             int64_t c, s;
             sincos_turn(T.d, t, &c, &s);
-            printf("%lld %lld %lld\n", (long long)c, (long long)s, (long long)cos_turn(T.d, t));
+            printf("%lld %lld\n", (long long)c, (long long)s);
         } else if (m == 't' && scanf("%la %la", &x, &q) == 2) {
             printf("%llu %llu\n", (unsigned long long)turns(x, split(turn_factor(q))),
                    (unsigned long long)turns((float)x, split(turn_factor(q))));
@@ -79,8 +79,7 @@ def test_sine_and_cosine(harness):
         int(a) << 32 | int(b) for a, b in rng.integers(0, 2**32, size=(4000, 2))]
     ts = [t % 2**64 for t in ts]
     worst = 0.0
-    for t, (c, s, c2) in zip(ts, harness([f"s {t}" for t in ts])):
-        assert c == c2
+    for t, (c, s) in zip(ts, harness([f"s {t}" for t in ts])):
         a = _turn_rad(t)
         worst = max(worst, abs(LD(int(c)) / LD(2) ** 62 - np.cos(a)),
                     abs(LD(int(s)) / LD(2) ** 62 - np.sin(a)))
