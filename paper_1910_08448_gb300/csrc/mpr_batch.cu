@@ -111,13 +111,11 @@ cudaError_t add_kernel(cudaGraphNode_t* node, cudaGraph_t body, const cudaGraphN
     return cudaGraphAddNode(node, body, dep, dep ? &ed : nullptr, dep ? 1 : 0, &np);
 }
 
-// Sweeps per turn of a loop: a turn of the conditional node costs about 6 us (17 problems of sides 64
+// The while loop of one group: a node of g without dependencies, so the groups' loops run side by side.
+// batch::kUnroll sweeps per turn: a turn of the conditional node costs about 6 us (17 problems of sides 64
 // ... 256: 61, 48, 46, 45 ms with 1, 4, 8, 16 sweeps a turn), a finished batch runs up to 7 empty sweeps
 // more. A red pass waits for the black pass before it by itself (pass_kernel), so every edge but the
 // loop's own is programmatic.
-constexpr int kUnroll = 8;
-
-// The while loop of one group: a node of g without dependencies, so the groups' loops run side by side.
 cudaError_t add_loop(cudaGraph_t g, const void* pass, size_t smem, int tiles, bool programmatic,
                      const batch::Args* args_dev, const PhiloxSched& keys)
 {
@@ -133,12 +131,12 @@ cudaError_t add_loop(cudaGraph_t g, const void* pass, size_t smem, int tiles, bo
     e = cudaGraphAddNode(&wnode, g, nullptr, nullptr, 0, &cp);
     if (e != cudaSuccess) return e;
     const cudaGraph_t body = cp.conditional.phGraph_out[0];
-    const int red = 0, black = 1, sweeps = kUnroll;
+    const int red = 0, black = 1, sweeps = batch::kUnroll;
     void* params_r[] = {&args_dev, const_cast<int*>(&red), const_cast<PhiloxSched*>(&keys)};
     void* params_b[] = {&args_dev, const_cast<int*>(&black), const_cast<PhiloxSched*>(&keys)};
     void* params_f[] = {&args_dev, &loop, const_cast<int*>(&sweeps)};
     cudaGraphNode_t last{}, next;
-    for (int i = 0; i < 2 * kUnroll && e == cudaSuccess; ++i) {
+    for (int i = 0; i < 2 * batch::kUnroll && e == cudaSuccess; ++i) {
         e = add_kernel(&next, body, i ? &last : nullptr, i > 0 && programmatic, pass, tiles, smem,
                        i & 1 ? params_b : params_r);
         last = next;

@@ -94,6 +94,7 @@ struct Args {
 struct Shape {
     int cols, rpt;
 };
+constexpr int kUnroll = 8;      // graph mode: sweeps per turn of a loop (see add_loop)
 constexpr int kMaxGroups = 8;   // graph mode: groups of problems, each with its own while loop
 constexpr int kShapes = 5;
 constexpr Shape kShape[kShapes] = {{128, 1}, {128, 2}, {128, 4}, {64, 1}, {64, 2}};

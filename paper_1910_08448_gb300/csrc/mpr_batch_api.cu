@@ -313,10 +313,7 @@ mpr_status launch_fill(mpr_batch_ctx* b, bool tune, int equil, int samples, floa
     A.qf = (float)b->opt.q;
     // round keys of the batch's seed for the tile kernels' parameter (counter parts unused)
     const PhiloxSched keys = philox_sched(0u, 0u, kTagMetropolis, 0u, A.seed_lo, A.seed_hi);
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    BCU(cudaEventCreate(&e0));
-    BCU(cudaEventCreate(&e1));
-    BCU(cudaEventRecord(e0, b->stream));
+    cudaGraphExec_t& ge = b->gexec[b->shape];
     if (active > 0) {
         if (!b->dArgs) BCHECK(balloc(b, &b->dArgs, batch::kMaxGroups * sizeof(batch::Args)));
         batch::Args all[batch::kMaxGroups];
@@ -328,23 +325,29 @@ mpr_status launch_fill(mpr_batch_ctx* b, bool tune, int equil, int samples, floa
         }
         BCU(cudaMemcpyAsync(b->dArgs, all, (size_t)ng * sizeof(batch::Args), cudaMemcpyHostToDevice,
                             b->stream));
-        if (b->use_graph == 2) {
-            cudaGraphExec_t& ge = b->gexec[b->shape];
-            const bool qhalf = A.qf == 0.5f;
-            if (ge && (b->gexec_tiles[b->shape] != b->ntiles || b->gexec_qhalf[b->shape] != qhalf)) {
-                cudaGraphExecDestroy(ge);
-                ge = nullptr;
-            }
-            if (!ge) {
-                BCU(batch_graph_build(b->prec.store, b->shape, ng, tiles, qhalf, b->dArgs, keys, &ge));
-                b->gexec_tiles[b->shape] = b->ntiles;
-                b->gexec_qhalf[b->shape] = qhalf;
-            }
-            BCU(cudaGraphLaunch(ge, b->stream));
-        } else {
+        // (built before the timed part: the autotuner compares launches)
+        const bool qhalf = A.qf == 0.5f;
+        if (b->use_graph == 2 && ge &&
+            (b->gexec_tiles[b->shape] != b->ntiles || b->gexec_qhalf[b->shape] != qhalf)) {
+            cudaGraphExecDestroy(ge);
+            ge = nullptr;
+        }
+        if (b->use_graph == 2 && !ge) {
+            BCU(batch_graph_build(b->prec.store, b->shape, ng, tiles, qhalf, b->dArgs, keys, &ge));
+            BCU(cudaGraphUpload(ge, b->stream));
+            b->gexec_tiles[b->shape] = b->ntiles;
+            b->gexec_qhalf[b->shape] = qhalf;
+        }
+    }
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    BCU(cudaEventCreate(&e0));
+    BCU(cudaEventCreate(&e1));
+    BCU(cudaEventRecord(e0, b->stream));
+    if (active > 0) {
+        if (b->use_graph == 2) BCU(cudaGraphLaunch(ge, b->stream));
+        else
             BCU(batch_launch(b->prec.store, b->shape, grid, b->dArgs, keys, b->stream,
                              b->use_graph != 0));
-        }
         b->launches += 1;
     }
     BCU(cudaEventRecord(e1, b->stream));
@@ -657,6 +660,7 @@ mpr_status mpr_batch_autotune(mpr_batch b, int sweeps, int* tile_rows_out, int* 
     if (!b) return bfail(MPR_ERR_INVALID_ARG, "batch is NULL");
     if (b->broken) return bfail(MPR_ERR_STATE, "the batch was left undefined by a device timeout");
     if (sweeps < 1) sweeps = 10;
+    sweeps = (sweeps + batch::kUnroll - 1) / batch::kUnroll * batch::kUnroll;   // whole turns of a loop
     long long total = 0;
     for (long long v : b->N) total += v;
     const auto key = std::make_tuple(b->n, total, b->prec.store, b->prec.energy);
