@@ -107,7 +107,10 @@ struct mpr_ctx {
     double prof_ms = 0.0;
     uint64_t prof_launches = 0, prof_pending_launches = 0;
 
-    // device memory
+    // device memory: two blocks (z, mask, part and scal; the state arrays), and what runs ask for
+    char* base = nullptr;
+    char* state = nullptr;
+    size_t base_bytes = 0, state_bytes = 0;
     double* z = nullptr;                 // N, row-major
     unsigned char* mask = nullptr;       // N, row-major
     void* ang[2] = {nullptr, nullptr};   // colour half-lattices, Ly x pitch, storage type
@@ -230,31 +233,101 @@ size_t mb_bytes(const mpr_ctx* h) { return (size_t)h->L.Ly * h->L.mpitch * 4; }
 size_t accd_bytes(const mpr_ctx* h) { return (size_t)h->L.Ly * h->L.pitch * 8; }
 size_t accf_bytes(const mpr_ctx* h) { return (size_t)h->L.Ly * h->L.pitch * 4; }
 
+// Pinned staging blocks of 16 doubles: kept for the next handle (at most kPinnedKeep of them) until
+// mpr_trim_memory. Pinning and unpinning a page took most of a small
+// handle's release (210 us, now 13) and, with a dozen allocations, half of its creation (400 us at 256^2,
+// now 200).
+constexpr size_t kPinnedKeep = 64;
+std::vector<double*> g_pinned;
+
+double* pinned_take()
+{
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        if (!g_pinned.empty()) {
+            double* const p = g_pinned.back();
+            g_pinned.pop_back();
+            return p;
+        }
+    }
+    double* p = nullptr;
+    return cudaHostAlloc(&p, 16 * sizeof(double), cudaHostAllocPortable) == cudaSuccess ? p : nullptr;
+}
+
+// The caller's stream has no copy to or from p in flight.
+void pinned_give(double* p)
+{
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        if (g_pinned.size() < kPinnedKeep) {
+            g_pinned.push_back(p);
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
+// Arrays of one device block, 256-byte aligned (the TMA maps and vector accesses ask for 16).
+struct Carve {
+    char* base;
+    size_t at = 0;
+    template <typename T> T* take(size_t bytes)
+    {
+        T* const p = base ? reinterpret_cast<T*>(base + at) : nullptr;
+        at += (bytes + 255) / 256 * 256;
+        return p;
+    }
+};
+
+// The state arrays of the handle's precision, in one block: angles and masks, then the sums (zeroed
+// at the start of a chain, from *sums on). base null: the size only.
+size_t carve_state(mpr_ctx* h, char* base, size_t* sums)
+{
+    Carve v{base};
+    for (int c = 0; c < 2; ++c) {
+        h->ang[c] = v.take<void>(ang_bytes(h));
+        h->mb[c] = v.take<uint32_t>(mb_bytes(h));
+    }
+    *sums = v.at;
+    const bool f64 = h->prec.acc == 0;
+    // (exact fixed-point partials of FP16 spins, tile kernel)
+    const bool fix = f64 && h->prec.store == kF16 && h->prec.func >= 1;
+    for (int c = 0; c < 2; ++c) {
+        h->acc[c] = f64 ? v.take<double>(accd_bytes(h)) : nullptr;
+        h->part32[c] = fix ? v.take<int>(accf_bytes(h)) : nullptr;
+        h->acc_hi[c] = f64 ? nullptr : v.take<float>(accf_bytes(h));
+        h->acc_lo[c] = f64 ? nullptr : v.take<float>(accf_bytes(h));
+    }
+    return v.at;
+}
+
 void free_state(mpr_ctx* h)
 {
+    dfree(h, &h->state, h->state_bytes);
+    h->state_bytes = 0;
     for (int c = 0; c < 2; ++c) {
-        dfree(h, &h->ang[c], ang_bytes(h));
-        dfree(h, &h->mb[c], mb_bytes(h));
-        dfree(h, &h->acc[c], accd_bytes(h));
-        dfree(h, &h->acc_hi[c], accf_bytes(h));
-        dfree(h, &h->acc_lo[c], accf_bytes(h));
-        dfree(h, &h->part32[c], accf_bytes(h));
+        h->ang[c] = nullptr;
+        h->mb[c] = nullptr;
+        h->acc[c] = nullptr;
+        h->acc_hi[c] = h->acc_lo[c] = nullptr;
+        h->part32[c] = nullptr;
     }
 }
 
 void free_all(mpr_ctx* h)
 {
     free_state(h);
-    dfree(h, &h->z, (size_t)h->N * 8);
-    dfree(h, &h->mask, (size_t)h->N);
-    dfree(h, &h->part, h->part_bytes);
-    dfree(h, &h->scal, 16 * 8);
+    dfree(h, &h->base, h->base_bytes);
+    h->z = nullptr;
+    h->mask = nullptr;
+    h->part = nullptr;
+    h->scal = nullptr;
     dfree(h, &h->eseries, (size_t)h->eseries_cap * 8);
     dfree(h, &h->tmpN, (size_t)h->N * 8);
     dfree(h, &h->halo, h->halo_bytes);
     dfree(h, &h->er, h->er_bytes);
     dfree(h, &h->rpart, h->rpart_bytes);
-    if (h->host) cudaFreeHost(h->host);
+    if (h->host) pinned_give(h->host);
     h->host = nullptr;
     if (h->ev0) cudaEventDestroy(h->ev0);
     if (h->ev1) cudaEventDestroy(h->ev1);
@@ -333,23 +406,12 @@ mpr_status init_state(mpr_ctx* h)
 {
     free_state(h);
     const Precision& p = h->prec;
-    for (int c = 0; c < 2; ++c) {
-        CHECK(dalloc(h, &h->ang[c], ang_bytes(h)));
-        CHECK(dalloc(h, &h->mb[c], mb_bytes(h)));
-        if (p.acc == 0) {
-            CHECK(dalloc(h, &h->acc[c], accd_bytes(h)));
-            CU(cudaMemsetAsync(h->acc[c], 0, accd_bytes(h), h->stream));
-            if (p.store == kF16 && p.func >= 1) {   // exact fixed-point partials (tile kernel)
-                CHECK(dalloc(h, &h->part32[c], accf_bytes(h)));
-                CU(cudaMemsetAsync(h->part32[c], 0, accf_bytes(h), h->stream));
-            }
-        } else {
-            CHECK(dalloc(h, &h->acc_hi[c], accf_bytes(h)));
-            CHECK(dalloc(h, &h->acc_lo[c], accf_bytes(h)));
-            CU(cudaMemsetAsync(h->acc_hi[c], 0, accf_bytes(h), h->stream));
-            CU(cudaMemsetAsync(h->acc_lo[c], 0, accf_bytes(h), h->stream));
-        }
-    }
+    size_t sums = 0;
+    const size_t need = carve_state(h, nullptr, &sums);
+    CHECK(dalloc(h, &h->state, need));
+    h->state_bytes = need;
+    carve_state(h, h->state, &sums);
+    CU(cudaMemsetAsync(h->state + sums, 0, need - sums, h->stream));
     h->nsplit = p.func != 0 ? split_tiles(h, false) : 0;
     h->nsplit_prop = p.func == 1 ? split_tiles(h, true) : 0;
     // Own rows of a plain pass with 16-bit spins: loaded at each row's update when both colours
@@ -415,6 +477,7 @@ mpr_status create_common(int Lx, int Ly, const double* values, const unsigned ch
     h->Nb = (long long)Lx * (Ly - 1) + (long long)Ly * (Lx - 1);
     auto bail = [&](mpr_status s) {
         std::string keep = g_err;
+        cudaStreamSynchronize(h->stream);   // no copy to the staging block is left
         free_all(h);
         delete h;
         g_err = keep;
@@ -422,7 +485,7 @@ mpr_status create_common(int Lx, int Ly, const double* values, const unsigned ch
     };
     mpr_status s;
     if (cudaGetDevice(&h->device) != cudaSuccess) return bail(fail(MPR_ERR_CUDA, "no CUDA device"));
-    if (cudaMallocHost(&h->host, 16 * sizeof(double)) != cudaSuccess)
+    if (!(h->host = pinned_take()))
         return bail(fail(MPR_ERR_OOM, "pinned host allocation failed"));
     const int nmm = 256;
     {
@@ -433,14 +496,22 @@ mpr_status create_common(int Lx, int Ly, const double* values, const unsigned ch
         for (size_t v : {a, b, c}) need = need > v ? need : v;
         h->part_bytes = need;
     }
-    if ((s = dalloc(h, &h->part, h->part_bytes)) != MPR_OK) return bail(s);
-    if ((s = dalloc(h, &h->scal, 16 * 8)) != MPR_OK) return bail(s);
+    auto carve = [&](char* base) {
+        Carve v{base};
+        h->scal = v.take<double>(16 * 8);
+        h->part = v.take<void>(h->part_bytes);
+        h->z = v.take<double>((size_t)h->N * 8);
+        h->mask = v.take<unsigned char>((size_t)h->N);
+        return v.at;
+    };
+    const size_t base_bytes = carve(nullptr);
+    if ((s = dalloc(h, &h->base, base_bytes)) != MPR_OK) return bail(s);
+    h->base_bytes = base_bytes;
+    carve(h->base);
     if (cudaMemsetAsync(h->scal, 0, 16 * 8, stream) != cudaSuccess ||
         cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
         return bail(fail(MPR_ERR_CUDA, "device query failed"));
     h->host[15] = 0.0;
-    if ((s = dalloc(h, &h->z, (size_t)h->N * 8)) != MPR_OK) return bail(s);
-    if ((s = dalloc(h, &h->mask, (size_t)h->N)) != MPR_OK) return bail(s);
     if (free_lattice) {
         if (cudaMemsetAsync(h->z, 0, (size_t)h->N * 8, stream) != cudaSuccess ||
             cudaMemsetAsync(h->mask, 0, (size_t)h->N, stream) != cudaSuccess)
@@ -770,6 +841,8 @@ void mpr_destroy(mpr_handle h)
 mpr_status mpr_trim_memory(void)
 {
     std::lock_guard<std::mutex> lock(g_pool_mu);
+    for (double* p : g_pinned) cudaFreeHost(p);
+    g_pinned.clear();
     for (cudaMemPool_t pool : g_pool) {
         if (!pool) continue;
         const cudaError_t e = cudaMemPoolTrimTo(pool, 0);
