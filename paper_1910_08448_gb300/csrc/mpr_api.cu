@@ -384,8 +384,9 @@ mpr_status validate_options(const mpr_options* o)
 // on S slots (resident blocks on the device).
 // - At most one wave: all of them, as the chain of a thread's rows and the uneven share of the SMs are
 //   what the pass costs (us per pass with none / all: 1500 x 2000 HDS 9.3 / 7.6, 2501 x 1333 BDS 9.5 / 8.1,
-//   2048^2 SDS 10.0 / 9.2, bounded HDS 12.0 / 10.8, 777 x 523 bounded 6.2 / 4.1). The kernels with
-//   fewer than four blocks per SM only where the halves fit one wave too (2501 x 1333 bounded SDS
+//   2048^2 SDS 10.0 / 9.2, bounded HDS 12.0 / 10.8, 777 x 523 bounded 6.2 / 4.1), unless the wave is full
+//   anyway (3107 x 1396 HDS, 572 tiles on 608 slots: 1 % slower). The kernels with fewer than four
+//   blocks per SM only where the halves fit one wave too (2501 x 1333 bounded SDS
 //   9.6 / 10.2, 1000 x 1700 DDS 9.0 / 9.7).
 // - Up to four waves of four blocks: the T mod S tiles of the partial one when twice as many fit a
 //   wave (4096^2 HDS 28.4 / 27.7, 2560^2 SDS 14.5 / 13.3), else half of them (3000^2 HDS 17.2 / 16.6).
@@ -395,7 +396,7 @@ int split_tiles(const mpr_ctx* h, bool bounded)
     const int per_sm = sweep_f32_plain_occupancy(h->prec, bounded), slots = per_sm * h->nsm;
     const int nt = sweep_f32_blocks(h->L);
     if (slots <= 0 || nt >= 16 * h->nsm) return 0;
-    if (nt <= slots) return per_sm >= 4 || 2 * nt <= slots ? nt : 0;
+    if (nt <= slots) return (per_sm >= 4 && 10 * nt <= 9 * slots) || 2 * nt <= slots ? nt : 0;
     const int rem = nt % slots;
     return 2 * rem <= slots ? rem : rem / 2;
 }
