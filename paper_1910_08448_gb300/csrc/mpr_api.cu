@@ -142,7 +142,7 @@ struct mpr_ctx {
     resident::Plan rplan{};
     unsigned long long* halo = nullptr;  // boundary rows in flight between blocks
     size_t halo_bytes = 0;
-    uint32_t epoch = 0;                  // tag of the last resident pass
+    uint32_t epoch = 0;                  // tags of resident launches so far (at most)
     float* er = nullptr;                 // row sums of measured sweeps
     void* rpart = nullptr;               // their tile partials
     size_t er_bytes = 0, rpart_bytes = 0;
@@ -362,7 +362,7 @@ mpr_status sync(mpr_ctx* h)
         CU(cudaMemsetAsync(dev_err(h), 0, sizeof(int), h->stream));
         CU(cudaStreamSynchronize(h->stream));
         return fail(e == MPR_ERR_DEVICE_TIMEOUT ? MPR_ERR_DEVICE_TIMEOUT : MPR_ERR_CUDA,
-                    "a device-side wait for a TMA copy ran out");
+                    "a device-side wait for a TMA copy or for a neighbouring block's rows ran out");
     }
     return harvest_profile(h);
 }
@@ -591,6 +591,10 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
     if (!p.cluster && !h->halo) {
         CHECK(ensure_scratch(h, &h->halo, &h->halo_bytes, resident::halo_bytes(p)));
         CU(cudaMemsetAsync(h->halo, 0, h->halo_bytes, h->stream));
+    }
+    if (h->epoch > 0x7FFFFFFFu) {   // tags start again: no word of an earlier launch may carry one
+        if (h->halo) CU(cudaMemsetAsync(h->halo, 0, h->halo_bytes, h->stream));
+        h->epoch = 0;
     }
     int most = n;
     if (measure) {
