@@ -585,6 +585,7 @@ mpr_status ensure_scratch(mpr_ctx* h, T** p, size_t* have, size_t bytes)
 mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
 {
     constexpr size_t kErBytes = 16u << 20;   // row sums of the measured sweeps of one launch
+    constexpr int kLongest = 4096;           // sweeps of a launch: 4 to 40 ms, then others get their turn
     const resident::Plan& p = h->rplan;
     const bool measure = (flags & kMeasure) != 0;
     *ran = true;
@@ -596,10 +597,10 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
         if (h->halo) CU(cudaMemsetAsync(h->halo, 0, h->halo_bytes, h->stream));
         h->epoch = 0;
     }
-    int most = n;
+    int most = std::min(n, kLongest);
     if (measure) {
         const size_t row = (size_t)h->L.Ly * p.G * 4, nt = (size_t)sweep_f32_blocks(h->L) * 8;
-        most = (int)std::min<size_t>((size_t)n, std::max<size_t>(3, kErBytes / row));
+        most = (int)std::min<size_t>((size_t)most, std::max<size_t>(3, kErBytes / row));
         CHECK(ensure_scratch(h, &h->er, &h->er_bytes, row * (size_t)most));
         CHECK(ensure_scratch(h, &h->rpart, &h->rpart_bytes, nt * (size_t)most));
     }

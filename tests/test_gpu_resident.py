@@ -125,3 +125,11 @@ def test_same_bits_for_every_plan(mpr, Lx, Ly, setup, q, acc):
     pr.mask[0, :2] = 1
     parts = ((2, 0), (3, 2), (0, 3), (1, 1), (25, 9))
     _same(_run(mpr, pr, setup, -1, q=q, acc=acc, parts=parts), _run(mpr, pr, setup, 0, q=q, acc=acc, parts=parts))
+
+
+@pytest.mark.parametrize("Lx,Ly", [(64, 64), (300, 211), (700, 500)])
+def test_more_sweeps_than_one_launch_takes(mpr, Lx, Ly):
+    """4096 sweeps a launch: the remainder of one sweep joins the launch before it."""
+    pr = mpr_inputs.make_problem(Lx, Ly, 0.6, field_seed=63, mask_seed=64, periodic=True)
+    parts = ((4097, 0), (8193, 4))
+    _same(_run(mpr, pr, "SDS", -1, parts=parts), _run(mpr, pr, "SDS", 0, parts=parts))
