@@ -643,7 +643,7 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
         a.epoch = p.cluster ? 0u : h->epoch;
         const cudaError_t e = resident::launch(p, h->prec.store, measure, sample, a.qf == 0.5f, a,
                                                h->stream);
-        if (e != cudaSuccess && k == 0) {
+        if (resident::too_large(e) && k == 0) {
             cudaGetLastError();
             h->rplan.nb = 0;
             *ran = false;

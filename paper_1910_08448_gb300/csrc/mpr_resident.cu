@@ -11,7 +11,6 @@ namespace resident {
 namespace {
 
 constexpr int kCluster = 16;                 // blocks of a cluster (non-portable size)
-constexpr size_t kSmem = 227 * 1024;         // shared memory of a block
 
 // Bands of equal height but one row pair, at most `most` of them: as few as the tallest allows.
 Plan bands(const Layout& L, int most)
@@ -41,7 +40,7 @@ Plan fine_plan(const Layout& L, int most, bool cluster, int depth)
     p.threads = 32 * (int)std::min<size_t>(warps, 64);
     p.smem = 2 * 4 * groups * 16 + (cluster ? (size_t)4 * halo_rows(depth) * 4 * G * 8 : 0) +
              4 * (size_t)(p.rows + 2 * depth) * (4 * G + 8) * 4;
-    return p.threads <= kFineThreads && p.smem <= kSmem ? p : Plan{};
+    return p.threads <= kFineThreads && p.smem <= kMaxSmem ? p : Plan{};
 }
 
 Plan coarse_plan(const Layout& L, int store, int most)
@@ -55,7 +54,7 @@ Plan coarse_plan(const Layout& L, int store, int most)
     // a second unit per thread only in bands taller than a pair: 5000 x 60 would leave most SMs idle and
     // take 5.7 us per pass (the tile kernel 4.1), 3500 x 600 takes 5.1 (6.0), 2300 x 1200 HDS 6.1 (9.1)
     if ((p.pair ? groups : 2 * one_role) > kCoarseThreads && p.rows == 2) return Plan{};
-    return p.smem <= kSmem ? p : Plan{};
+    return p.smem <= kMaxSmem ? p : Plan{};
 }
 
 // Tile (tx, ty) of a measured black pass: the thread's rows in the tile kernel's order, its warps by

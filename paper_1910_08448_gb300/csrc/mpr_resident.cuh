@@ -658,7 +658,10 @@ cudaError_t go_shape(const Plan& p, const Args& a, cudaStream_t st)
                                : p.fine  ? fine_kernel<S, MEASURE, SAMPLE, QM, false>
                                : p.pair  ? coarse_kernel<S, MEASURE, SAMPLE, QM, true>
                                          : coarse_kernel<S, MEASURE, SAMPLE, QM, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    // An attribute belongs to the function, and handles of other host threads launch it too: always the same
+    // value, the most a plan takes. (With p.smem here, a smaller lattice's value that landed between
+    // a larger one's call and its launch made that launch fail.)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(p.nb);

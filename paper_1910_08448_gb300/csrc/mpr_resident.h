@@ -9,6 +9,7 @@ namespace resident {
 
 constexpr int kFineThreads = 768;
 constexpr int kCoarseThreads = 512;
+constexpr size_t kMaxSmem = 227 * 1024;   // dynamic shared memory of a block, at most
 
 // How a lattice is laid out over the blocks of the launch.
 struct Plan {
@@ -56,6 +57,12 @@ size_t halo_bytes(const Plan& p);
 // nsweeps hybrid sweeps; sample: 0 none, 1 FP64 sums, 2 Kahan sums (only with measure).
 cudaError_t launch(const Plan& p, int store, bool measure, int sample, bool qhalf, const Args& a,
                    cudaStream_t st);
+// The launch was refused because the device cannot hold its blocks at once (nothing ran).
+inline bool too_large(cudaError_t e)
+{
+    return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
+           e == cudaErrorLaunchOutOfResources;
+}
 // out[k] = the fixed-order sum of the n partials of sweep k (reduce_kernel's order), a block per sweep.
 cudaError_t launch_sums(const void* part, int n, int nsweeps, bool e32, double* out, cudaStream_t st);
 // The raw bond sums of nsweeps measured sweeps from their row sums, in the summation order of the

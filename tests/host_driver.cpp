@@ -1,0 +1,77 @@
+// The host driver of libmpr on the stand-in runtime (fake_cudart.cpp); test_host_driver.py builds it,
+// names a scenario and reads what is printed: the status of the call, then the launches in order.
+#include <cuda_runtime.h>
+#include <stdio.h>
+#include <stdlib.h>
+#include <string.h>
+
+#include <thread>
+
+#include "fake_cudart.h"
+#include "mpr.h"
+
+namespace {
+
+mpr_handle handle(int Lx, int Ly)
+{
+    std::vector<double> z((size_t)Lx * Ly, 0.5);
+    std::vector<unsigned char> m((size_t)Lx * Ly, 1);
+    mpr_handle h = nullptr;
+    if (mpr_create(Lx, Ly, z.data(), m.data(), &h) != MPR_OK || mpr_set_temperature(h, 0.1) != MPR_OK) {
+        fprintf(stderr, "%s\n", mpr_last_error());
+        exit(1);
+    }
+    return h;
+}
+
+bool is_resident(const fake::Launch& l)
+{
+    return l.name.find("fine_kernel") != std::string::npos || l.name.find("coarse_kernel") != std::string::npos;
+}
+
+void report(mpr_status s)
+{
+    printf("status %d\n", (int)s);
+    for (const fake::Launch& l : fake::launches)
+        printf("%s programmatic=%d cooperative=%d smem=%zu\n", l.name.c_str(), l.programmatic, l.cooperative, l.smem);
+}
+
+}  // namespace
+
+int main(int argc, char** argv)
+{
+    const char* const what = argc > 1 ? argv[1] : "";
+    auto num = [&](int i) { return i < argc ? atoi(argv[i]) : 0; };
+    if (!strcmp(what, "run")) {   // Lx Ly equil samples
+        mpr_handle h = handle(num(2), num(3));
+        fake::launches.clear();
+        report(mpr_run(h, num(4), num(5)));
+        mpr_destroy(h);
+    } else if (!strcmp(what, "other")) {   // Lx Ly, and Lx Ly of a handle that runs before each resident launch
+        mpr_handle h = handle(num(2), num(3)), g = handle(num(4), num(5));
+        fake::launches.clear();
+        bool inside = false;
+        fake::on_launch = [&](const fake::Launch& l) {
+            if (inside || !is_resident(l)) return 0;
+            inside = true;
+            mpr_status s = MPR_OK;
+            std::thread([&] { s = mpr_run(g, 50, 0); }).join();
+            inside = false;
+            return s == MPR_OK ? 0 : (int)cudaErrorUnknown;
+        };
+        report(mpr_run(h, 50, 40));
+        fake::on_launch = nullptr;
+        mpr_destroy(h);
+        mpr_destroy(g);
+    } else if (!strcmp(what, "refuse")) {   // Lx Ly, error code of the resident launches
+        mpr_handle h = handle(num(2), num(3));
+        fake::launches.clear();
+        fake::on_launch = [&](const fake::Launch& l) { return is_resident(l) ? num(4) : 0; };
+        report(mpr_run(h, 5, 4));
+        fake::on_launch = nullptr;
+        mpr_destroy(h);
+    } else {
+        return 2;
+    }
+    return 0;
+}

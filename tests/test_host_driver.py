@@ -1,0 +1,75 @@
+"""The library's host code on a stand-in CUDA runtime, on the CPU: which launches a call makes, in which
+order and with which attributes, and what it does when a launch or an allocation is refused.
+"""
+import glob
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+HERE = os.path.join(ROOT, "tests")
+
+
+@pytest.fixture(scope="module")
+def driver(tmp_path_factory):
+    import __graft_entry__
+    from paper_1910_08448_gb300 import _build
+
+    __graft_entry__.build()
+    objs = sorted(glob.glob(os.path.join(_build.BUILD, "mpr_*.o")))
+    if len(objs) != len(_build.sources()):   # a library that was built elsewhere
+        _build.build(force=True)
+        objs = sorted(glob.glob(os.path.join(_build.BUILD, "mpr_*.o")))
+    exe = str(tmp_path_factory.mktemp("driver") / "driver")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(_build.nvcc())), "include")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-I", cuda, "-I", _build.INCLUDE, "-I", HERE,
+                    os.path.join(HERE, "host_driver.cpp"), os.path.join(HERE, "fake_cudart.cpp"), *objs,
+                    "-ldl", "-lpthread", "-o", exe], check=True)
+
+    def run(*args):
+        r = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, timeout=120)
+        assert r.returncode == 0, (r.returncode, r.stderr)
+        lines = r.stdout.strip().split("\n")
+        out = []
+        for ln in lines[1:]:
+            name, *rest = ln.split()
+            out.append((name, {k: int(v) for k, v in (p.split("=") for p in rest)}))
+        return int(lines[0].split()[1]), out
+
+    return run
+
+
+def _resident(name):
+    return "fine_kernel" in name or "coarse_kernel" in name
+
+
+def _tile(name):
+    return "sweep_f32_kernel" in name
+
+
+# a larger lattice whose resident kernel is also the smaller one's (row pairs; one row; a grid of the
+# fine kernel), and another handle's thread that runs in between
+@pytest.mark.parametrize("big,small", [((1400, 1200), (1024, 1024)), ((777, 523), (700, 400)),
+                                       ((300, 300), (200, 150))])
+def test_a_smaller_lattice_leaves_the_shared_memory_of_a_larger_one(driver, big, small):
+    status, calls = driver("other", *big, *small)
+    assert status == 0
+    names = [n for n, _ in calls]
+    most = max(a["smem"] for n, a in calls if _resident(n))
+    mine = [n for n, a in calls if _resident(n) and a["smem"] == most]
+    assert len(mine) >= 2 and not any(_tile(n) for n in names)
+
+
+REFUSED = {"cooperative launch too large": 720, "invalid cluster size": 912, "out of resources": 701}
+OTHER = {"invalid value": 1, "invalid configuration": 9, "unknown": 999}
+
+
+@pytest.mark.parametrize("shape", [(64, 64), (300, 300), (777, 523)])
+def test_only_a_launch_that_is_too_large_falls_back(driver, shape):
+    for code in REFUSED.values():
+        status, calls = driver("refuse", *shape, code)
+        assert status == 0 and sum(_tile(n) for n, _ in calls) == 2 * 9
+    for code in OTHER.values():
+        status, calls = driver("refuse", *shape, code)
+        assert status == 5 and not any(_tile(n) for n, _ in calls)
