@@ -143,6 +143,7 @@ struct mpr_ctx {
     unsigned long long* halo = nullptr;  // boundary rows in flight between blocks
     size_t halo_bytes = 0;
     uint32_t epoch = 0;                  // tags of resident launches so far (at most)
+    bool after_resident = false;         // the last kernel that wrote the angles is a resident one
     float* er = nullptr;                 // row sums of measured sweeps
     void* rpart = nullptr;               // their tile partials
     size_t er_bytes = 0, rpart_bytes = 0;
@@ -650,6 +651,7 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
             return MPR_OK;
         }
         CU(e);
+        h->after_resident = true;
         if (measure)
             CU(resident::launch_energies(h->L, h->prec.energy == 1, h->er, m, h->rpart,
                                          h->eseries + k, h->stream));
@@ -737,6 +739,8 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
             a.acc_hi = h->acc_hi[c];
             a.part32 = h->part32[c];
             a.acc_lo = h->acc_lo[c];
+            a.after_all = h->after_resident ? 1 : 0;
+            h->after_resident = false;
             if (kind == 1 && h->stall_ns > 0) {   // injected stall: this launch only
                 SweepArgs s = a;
                 s.stall_test = 1;

@@ -74,6 +74,8 @@ struct SweepArgs {
                                    // prediction sites are added here (NULL: not counted)
     int nsplit;                // one-tile-per-block FP32 kernel, plain passes: the last nsplit
                                // tiles run as two half-height tiles each (0: none)
+    int after_all;             // the kernel in front of this pass on the stream is no pass and wrote
+                               // this pass's own colour: not launched as its programmatic dependent
     int late;                  // same kernel, plain passes with 16-bit spins: 1 = load each own
                                // row just before its update (the state is resident in L2), 0 =
                                // load all own rows before the staging

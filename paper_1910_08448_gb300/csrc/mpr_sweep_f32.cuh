@@ -88,7 +88,9 @@ __global__ void __launch_bounds__(256, sizeof(S) == 8 ? 2
 }
 
 // Launched as a programmatic dependent launch: while the previous pass's last blocks finish, this
-// pass's blocks are scheduled and load their own rows (see sweep_tile).
+// pass's blocks are scheduled and load their own rows (see sweep_tile). Not behind a resident launch
+// (a.after_all), whose last stores are both colours: only the wait makes them visible, and the own rows are
+// loaded before it.
 template <typename S, bool MEASURE, int SAMPLE, bool PROP, int QM, bool HM>
 cudaError_t go_q(const SweepArgs& a, cudaStream_t st)
 {
@@ -102,7 +104,7 @@ cudaError_t go_q(const SweepArgs& a, cudaStream_t st)
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = a.after_all ? 0 : 1;
     if constexpr (!MEASURE && SAMPLE == 0 && !PROP && sizeof(S) == 2) {
         if (a.late) return cudaLaunchKernelEx(&cfg, sweep_f32_kernel<S, kRows, false, 0, false, QM, HM, true>, a);
     }

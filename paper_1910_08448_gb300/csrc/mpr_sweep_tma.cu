@@ -252,7 +252,7 @@ cudaError_t go_tma_q(const SweepArgs& a, const TmaMaps& m, int nsm, cudaStream_t
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = a.after_all ? 0 : 1;   // (the own colour's copy is issued before the wait)
     return cudaLaunchKernelEx(&cfg, kern, b, m.other[c ^ 1], m.own[c], m.mask[c]);
 }
 

@@ -753,7 +753,8 @@ __device__ __forceinline__ void count_accepted(int n_acc, unsigned long long* co
 // PDL (programmatic dependent launch, one tile per block): the block reads its own colour's values
 // and bits, then waits for the previous kernel (the other colour's pass), then lets the next
 // kernel in the stream start launching. The own colour was last written two passes back, which
-// has completed: the previous pass's blocks released this pass only after their own wait.
+// has completed: the previous pass's blocks released this pass only after their own wait. (Behind any other
+// kernel that wrote it, the pass is launched without the attribute: SweepArgs::after_all.)
 // Everything the previous pass may write (the other colour, accumulators, energy partials) is
 // touched only after the wait.
 // PROP: bounded proposals of half-width *a.width; accepted ones counted into *a.accepted.

@@ -47,6 +47,14 @@ int main(int argc, char** argv)
         fake::launches.clear();
         report(mpr_run(h, num(4), num(5)));
         mpr_destroy(h);
+    } else if (!strcmp(what, "tune")) {   // Lx Ly n_eq n_meas
+        mpr_handle h = handle(num(2), num(3));
+        mpr_tuning t{num(4), num(5), 0.1, 1.0, 0.0, 1.5, 4};
+        mpr_set_tuning(h, &t);
+        fake::launches.clear();
+        double T;
+        report(mpr_tune_temperature(h, &T));
+        mpr_destroy(h);
     } else if (!strcmp(what, "other")) {   // Lx Ly, and Lx Ly of a handle that runs before each resident launch
         mpr_handle h = handle(num(2), num(3)), g = handle(num(4), num(5));
         fake::launches.clear();

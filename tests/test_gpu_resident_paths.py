@@ -89,3 +89,21 @@ def test_two_sizes_on_two_threads(mpr, shapes):
     for g, w in zip(got, want):
         assert np.array_equal(g[0], w[0]) and np.array_equal(g[1], w[1])
         assert g[2] == n * (1 + 3) and w[2] == n * (4 + 5)
+
+
+# one sweep behind a resident launch, which runs the tile kernel: on a cluster, a grid every 4 and 2 passes,
+# rows and row pairs
+@pytest.mark.parametrize("Lx,Ly", [(64, 64), (128, 127), (90, 767), (400, 300), (777, 523), (1400, 1200)])
+@pytest.mark.parametrize("setup", ["SDS", "HDS", "BSS"])
+def test_one_sweep_behind_a_resident_launch(mpr, Lx, Ly, setup):
+    pr, out = _problem(Lx, Ly), []
+    for kind in (-1, 0):
+        h = _handle(mpr, pr, setup, kind)
+        try:
+            for equil in (2, 25, 3, 4097, 7):
+                mpr.mpr_run(h, equil, 1)
+            out.append((mpr.mpr_get_state(h)[0], mpr.mpr_predict(h), mpr.mpr_get_info(h)["e_bond_mean"]))
+        finally:
+            mpr.mpr_destroy(h)
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    assert out[0][2] == out[1][2]

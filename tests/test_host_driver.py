@@ -73,3 +73,16 @@ def test_only_a_launch_that_is_too_large_falls_back(driver, shape):
     for code in OTHER.values():
         status, calls = driver("refuse", *shape, code)
         assert status == 5 and not any(_tile(n) for n, _ in calls)
+
+
+# one sweep behind a resident launch: its first pass loads its own rows before it waits for the kernel in
+# front, and the resident kernel wrote both colours
+@pytest.mark.parametrize("shape", [(64, 64), (300, 300), (777, 523), (1400, 1200)])
+def test_a_pass_behind_a_resident_launch_is_no_programmatic_dependent(driver, shape):
+    for call in (("run", *shape, 2, 1), ("run", *shape, 25, 1), ("run", *shape, 4097, 1), ("tune", *shape, 3, 1)):
+        status, calls = driver(*call)
+        behind = [i for i in range(1, len(calls)) if _tile(calls[i][0]) and not _tile(calls[i - 1][0])]
+        assert status in (0, 4) and behind and all(_resident(calls[i - 1][0]) for i in behind)
+        for i in behind:
+            assert calls[i][1]["programmatic"] == 0
+            assert _tile(calls[i + 1][0]) and calls[i + 1][1]["programmatic"] == 1   # the black pass may
