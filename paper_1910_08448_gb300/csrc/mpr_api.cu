@@ -491,7 +491,7 @@ mpr_status create_common(int Lx, int Ly, const double* values, const unsigned ch
         return bail(fail(MPR_ERR_OOM, "pinned host allocation failed"));
     const int nmm = 256;
     {
-        size_t need = 0;
+        size_t need = (size_t)std::max(sweep_blocks(h->L, h->prec), sweep_f32_blocks(h->L)) * 8;
         size_t a = (size_t)sample_energy_blocks(h->L) * 16;
         size_t b = (size_t)energy_blocks(h->L) * 8;
         size_t c = (size_t)nmm * 32;
@@ -568,30 +568,37 @@ mpr_status fold_partials(mpr_ctx* h)
     return MPR_OK;
 }
 
-// A scratch array of at least `bytes`.
+// A scratch array of at least `bytes`. No memory for it is no error (*got = false): every run that uses
+// scratch can do without, so it needs no more memory than the handle has had since its creation.
 template <typename T>
-mpr_status ensure_scratch(mpr_ctx* h, T** p, size_t* have, size_t bytes)
+mpr_status ensure_scratch(mpr_ctx* h, T** p, size_t* have, size_t bytes, bool* got)
 {
+    *got = true;
     if (bytes <= *have) return MPR_OK;
     dfree(h, p, *have);
     *have = 0;
-    CHECK(dalloc(h, p, bytes));
+    const mpr_status s = dalloc(h, p, bytes);
+    if (s == MPR_ERR_OOM) {
+        *got = false;
+        return MPR_OK;
+    }
+    CHECK(s);
     *have = bytes;
     return MPR_OK;
 }
 
 // n sweeps by the resident kernel, as few launches as the scratch of measured sweeps allows.
-// *ran = false when the device cannot hold the launch's blocks at once: nothing has changed then,
-// and the handle's later sweeps run one launch per pass.
+// *ran = false, and nothing has changed, when there is no memory for its scratch, or when the device cannot
+// hold the launch's blocks at once (then the handle's later sweeps run one launch per pass too).
 mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
 {
     constexpr size_t kErBytes = 16u << 20;   // row sums of the measured sweeps of one launch
     constexpr int kLongest = 4096;           // sweeps of a launch: 4 to 40 ms, then others get their turn
     const resident::Plan& p = h->rplan;
     const bool measure = (flags & kMeasure) != 0;
-    *ran = true;
-    if (!p.cluster && !h->halo) {
-        CHECK(ensure_scratch(h, &h->halo, &h->halo_bytes, resident::halo_bytes(p)));
+    if (resident::halo_bytes(p) > h->halo_bytes) {
+        CHECK(ensure_scratch(h, &h->halo, &h->halo_bytes, resident::halo_bytes(p), ran));
+        if (!*ran) return MPR_OK;
         CU(cudaMemsetAsync(h->halo, 0, h->halo_bytes, h->stream));
     }
     if (h->epoch > 0x7FFFFFFFu) {   // tags start again: no word of an earlier launch may carry one
@@ -602,8 +609,9 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
     if (measure) {
         const size_t row = (size_t)h->L.Ly * p.G * 4, nt = (size_t)sweep_f32_blocks(h->L) * 8;
         most = (int)std::min<size_t>((size_t)most, std::max<size_t>(3, kErBytes / row));
-        CHECK(ensure_scratch(h, &h->er, &h->er_bytes, row * (size_t)most));
-        CHECK(ensure_scratch(h, &h->rpart, &h->rpart_bytes, nt * (size_t)most));
+        CHECK(ensure_scratch(h, &h->er, &h->er_bytes, row * (size_t)most, ran));
+        if (*ran) CHECK(ensure_scratch(h, &h->rpart, &h->rpart_bytes, nt * (size_t)most, ran));
+        if (!*ran) return MPR_OK;
     }
     resident::Args a{};
     a.Lx = h->L.Lx;
@@ -708,7 +716,7 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
         CU(cudaEventRecord(h->ev0, h->stream));
     }
     if (h->rplan.nb > 0 && n >= 2 && h->sweep_force < 0 && !h->prop_on) {
-        bool ran = false;
+        bool ran = true;
         CHECK(resident_sweeps(h, n, T, flags, &ran));
         if (ran) {
             if (flags == 0 && n >= 2 * (1 + kCalSweeps) && h->sweep_kind < 0) h->sweep_kind = 0;
@@ -723,12 +731,16 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
     // measured sweeps: the energy partials of up to `most` sweeps, then one launch sums them all (one
     // small launch after every sweep kept the next pass from starting: 4 us of each)
     const size_t epart = (size_t)nblk * (h->prec.energy == 1 ? 4 : 8);
-    const int most = (int)std::min<size_t>((size_t)n, std::max<size_t>(1, ((size_t)4 << 20) / epart));
-    if (flags & kMeasure) CHECK(ensure_scratch(h, &h->rpart, &h->rpart_bytes, epart * (size_t)most));
+    // (without memory for that: sweep by sweep, in the handle's own partials)
+    int most = (int)std::min<size_t>((size_t)n, std::max<size_t>(1, ((size_t)4 << 20) / epart));
+    bool got = true;
+    if (flags & kMeasure) CHECK(ensure_scratch(h, &h->rpart, &h->rpart_bytes, epart * (size_t)most, &got));
+    if (!got) most = 1;
+    char* const parts = static_cast<char*>(got ? h->rpart : h->part);
     // one hybrid sweep (both colour passes) with kernel kind (0/1; ignored for FP64 functions)
     auto one = [&](int k, int kind) -> mpr_status {
         a.sweep = h->sweep;
-        if (flags & kMeasure) a.epart = static_cast<char*>(h->rpart) + (size_t)(k % most) * epart;
+        if (flags & kMeasure) a.epart = parts + (size_t)(k % most) * epart;
         for (int c = 0; c < 2; ++c) {
             a.colour = c;
             a.ph = philox_sched(a.sweep, a.problem, kTagMetropolis, (uint32_t)c, a.seed_lo, a.seed_hi);
@@ -755,7 +767,7 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
         }
         const bool sum = (flags & kMeasure) && (k % most == most - 1 || k + 1 == n);
         if (sum)
-            CU(resident::launch_sums(h->rpart, nblk, k % most + 1, h->prec.energy == 1,
+            CU(resident::launch_sums(parts, nblk, k % most + 1, h->prec.energy == 1,
                                      h->eseries + (k - k % most), h->stream));
         if (adapt) CU(launch_adapt_width(h->scal + 14, prop_count(h), h->Np, h->prop_target, h->stream));
         h->launches += 2 + (sum ? 1 : 0) + (adapt ? 1 : 0);

@@ -47,6 +47,21 @@ int main(int argc, char** argv)
         fake::launches.clear();
         report(mpr_run(h, num(4), num(5)));
         mpr_destroy(h);
+    } else if (!strcmp(what, "scarce")) {   // Lx Ly equil samples func: no allocation above 300 bytes
+        mpr_handle h = handle(num(2), num(3));
+        mpr_options o;
+        mpr_get_options(h, &o);
+        o.func = num(6);
+        if (mpr_set_options(h, &o) != MPR_OK || mpr_set_temperature(h, 0.1) != MPR_OK) return 1;
+        mpr_info before, after;
+        mpr_get_info(h, &before);
+        fake::launches.clear();
+        fake::alloc_limit = 300;
+        const mpr_status s = mpr_run(h, num(4), num(5));
+        mpr_get_info(h, &after);
+        report(s);
+        if (!fake::refused_allocs || after.device_bytes > before.device_bytes + 300) return 1;
+        mpr_destroy(h);
     } else if (!strcmp(what, "tune")) {   // Lx Ly n_eq n_meas
         mpr_handle h = handle(num(2), num(3));
         mpr_tuning t{num(4), num(5), 0.1, 1.0, 0.0, 1.5, 4};

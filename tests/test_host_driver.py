@@ -86,3 +86,16 @@ def test_a_pass_behind_a_resident_launch_is_no_programmatic_dependent(driver, sh
         for i in behind:
             assert calls[i][1]["programmatic"] == 0
             assert _tile(calls[i + 1][0]) and calls[i + 1][1]["programmatic"] == 1   # the black pass may
+
+
+# no memory for boundary rows, row sums or partials (mpr_run gave MPR_ERR_OOM): one launch per pass, the energy
+# partials of each sweep summed before the next
+@pytest.mark.parametrize("shape", [(100, 80), (300, 300), (777, 523), (1400, 1200), (4096, 300)])
+@pytest.mark.parametrize("func", [0, 1])
+def test_runs_without_memory_for_scratch(driver, shape, func):
+    status, calls = driver("scarce", *shape, 5, 30, func)
+    assert status == 0
+    sums = [i for i, (n, _) in enumerate(calls) if "sweep_sums_kernel" in n]
+    passes = [i for i, (n, _) in enumerate(calls) if _tile(n) or "12sweep_kernel" in n]
+    assert len(sums) == 30 and all(len([p for p in passes if p < s]) % 2 == 0 for s in sums)
+    assert len(passes) + 2 * sum(_resident(n) for n, _ in calls) * 5 == 2 * 35
