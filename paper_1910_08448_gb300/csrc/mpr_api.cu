@@ -493,7 +493,7 @@ mpr_status create_common(int Lx, int Ly, const double* values, const unsigned ch
     {
         size_t need = (size_t)std::max(sweep_blocks(h->L, h->prec), sweep_f32_blocks(h->L)) * 8;
         size_t a = (size_t)sample_energy_blocks(h->L) * 16;
-        size_t b = (size_t)energy_blocks(h->L) * 8;
+        size_t b = (size_t)energy_blocks(h->L) * 16;
         size_t c = (size_t)nmm * 32;
         for (size_t v : {a, b, c}) need = need > v ? need : v;
         h->part_bytes = need;

@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
     const int lane = threadIdx.x & 31;
     const int nsx = (L.Lxh + 29) / 30;
     const long long nstrips = (long long)nsx * ((L.Ly + rows - 1) / rows);
-    double sum = 0.0;
+    energy::Sum sum{0.0, 0.0};
     for (long long st = (long long)blockIdx.x * energy::kWarpsPerBlock + (threadIdx.x >> 5);
          st < nstrips; st += (long long)gridDim.x * energy::kWarpsPerBlock) {
         const int sy = (int)(st / nsx), sx = (int)(st - (long long)sy * nsx);
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
         V fu = red_at(y0 - 1), fm = red_at(y0);
         bool oku = fixed::in_range(fu), okm = fixed::in_range(fm);
         energy::Vec uu = unit_at(y0 - 1, fu), um = unit_at(y0, fm);
-        int64_t acc = 0;   // at most 16 terms of 2^52
+        int64_t acc = 0;   // at most 16 terms of 2^58
         for (int y = y0; y < y1; ++y) {
             const V fd = red_at(y + 1);
             const bool okd = fixed::in_range(fd);
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
                     if (y > 0) { sincos(q * (double)fu, &sn, &cs); hx += cs; hy += sn; }
                     if (y + 1 < L.Ly) { sincos(q * (double)fd, &sn, &cs); hx += cs; hy += sn; }
                     sincos(q * (double)fb, &sn, &cs);
-                    sum += cs * hx + sn * hy;
+                    sum.add_fp64(cs * hx + sn * hy);
                 }
             }
             fu = fm;
@@ -271,27 +271,16 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
             oku = okm;
             okm = okd;
         }
-        sum += (double)acc * energy::kTermUnit;
+        sum.add(acc);
     }
-    const double s = energy::block_sum(sum);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    energy::block_sum(sum, part);
 }
 
-// Fixed-order sum of n partials: thread t adds entries t, t + 256, ... then a tree in shared memory.
-template <typename E>
-__global__ void __launch_bounds__(kThreads) reduce_kernel(const E* __restrict__ part, int n,
-                                                          double* __restrict__ out)
+__global__ void __launch_bounds__(kThreads) energy_final(const double* __restrict__ part, int n,
+                                                         double* __restrict__ out)
 {
-    __shared__ E ss[kThreads];
-    E s = (E)0;
-    for (int i = threadIdx.x; i < n; i += kThreads) s += part[i];
-    ss[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = kThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) ss[threadIdx.x] += ss[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = (double)ss[0];
+    const double s = energy::final_sum(part, n);
+    if (threadIdx.x == 0) *out = s;
 }
 
 // --------------------------------------------------------------------------------------------
@@ -497,7 +486,7 @@ cudaError_t launch_energy_fp64(const Layout& L, const Precision& p, const void* 
         energy_kernel<S><<<nblk, kThreads, 0, st>>>(L, static_cast<const S*>(ang0),
                                                     static_cast<const S*>(ang1), q,
                                                     fixed::turn_factor(q), energy_rows(L), part);
-        reduce_kernel<double><<<1, kThreads, 0, st>>>(part, nblk, out);
+        energy_final<<<1, kThreads, 0, st>>>(part, nblk, out);
         return cudaGetLastError();
     });
 }

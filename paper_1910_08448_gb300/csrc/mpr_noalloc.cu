@@ -24,13 +24,13 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr long long kMaxSites = 1ll << 28;    // 16384 x 16384
-constexpr int kMaxBlocks = 4096;              // partial sums of the first pass
+constexpr int kPartials = 4096;               // words of the first pass's partial sums
 constexpr int kMaxDevices = 64;
 
-// The scratch: one partial sum per block of the first pass. Every block of a call writes its own
+// The scratch: two words per block of the first pass (energy::Sum). Every block of a call writes its own
 // slot before the second pass reads it, so nothing has to be cleared between calls. Calls that
 // overlap on the GPU (for example on two streams) use the same slots and race.
-static __device__ __align__(256) double g_bond_partials[kMaxBlocks];
+static __device__ __align__(256) double g_bond_partials[kPartials];
 
 // First pass: sums of cos[q(phi_s - phi_right)] and cos[q(phi_s - phi_down)] (Eq. 2, open
 // boundaries). A strip is 31 columns x `rows` rows of one warp, lane 31 holding the right
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kThreads) bond_partials(int Lx, int Ly, int ro
     const int lane = threadIdx.x & 31;
     const int nsx = (Lx + 30) / 31;
     const long long nstrips = (long long)nsx * ((Ly + rows - 1) / rows);
-    double sum = 0.0;
+    energy::Sum sum{0.0, 0.0};
     for (long long st = (long long)blockIdx.x * energy::kWarpsPerBlock + (threadIdx.x >> 5);
          st < nstrips; st += (long long)gridDim.x * energy::kWarpsPerBlock) {
         const int sy = (int)(st / nsx), sx = (int)(st - (long long)sy * nsx);
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kThreads) bond_partials(int Lx, int Ly, int ro
         double f = has ? *p : 0.0, fb = 0.0;
         energy::Vec u = energy::unit_of_turn(tab, energy::turns_signed(f, k)), ub;
         bool ok = energy::in_range_signed(f), okb;
-        int64_t acc = 0;   // at most 16 terms of 2^51
+        int64_t acc = 0;   // at most 16 terms of 2^57
         for (int y = y0; y < y1; ++y) {
             const bool below = y + 1 < Ly;
             p += Lx;
@@ -74,33 +74,24 @@ __global__ void __launch_bounds__(kThreads) bond_partials(int Lx, int Ly, int ro
                 acc += mine ? e : 0;
             } else {
                 const double fr = __shfl_down_sync(0xffffffffu, f, 1);
-                if (right) sum += cos(q * (f - fr));
-                if (mine && below) sum += cos(q * (f - fb));
+                if (right) sum.add_fp64(cos(q * (f - fr)));
+                if (mine && below) sum.add_fp64(cos(q * (f - fb)));
             }
             f = fb;
             u = ub;
             ok = okb;
         }
-        sum += (double)acc * energy::kTermUnit;
+        sum.add(acc);
     }
-    const double s = energy::block_sum(sum);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    energy::block_sum(sum, part);
 }
 
 // Second pass, one block: fixed-order sum of the partials, e_b = -sum / N_b.
 __global__ void __launch_bounds__(kThreads) bond_final(const double* __restrict__ part, int nblk,
                                                        double n_bonds, double* __restrict__ out)
 {
-    __shared__ double sh[kThreads];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < nblk; i += kThreads) s += part[i];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = kThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *out = -sh[0] / n_bonds;
+    const double s = mpr::energy::final_sum(part, nblk);
+    if (threadIdx.x == 0) *out = -s / n_bonds;
 }
 
 // Device address of g_bond_partials per device. In host code the array's name only stands for
@@ -157,7 +148,7 @@ extern "C" mpr_status mpr_bond_energy_noalloc(int Lx, int Ly, const double* angl
     const int nsx = (Lx + 30) / 31, rows = mpr::energy::strip_rows(nsx, Ly);
     const long long strips = (long long)nsx * ((Ly + rows - 1) / rows);
     const int nblk = (int)std::min<long long>((strips + 7) / 8, 152 * 6);
-    static_assert(152 * 6 <= kMaxBlocks, "one partial per block");
+    static_assert(2 * 152 * 6 <= kPartials, "two words per block");
     const double n_bonds = (double)Lx * (Ly - 1) + (double)Ly * (Lx - 1);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     bond_partials<<<nblk, kThreads, 0, st>>>(Lx, Ly, rows, angles_dev, q,

@@ -89,7 +89,8 @@ __global__ void __launch_bounds__(256) tile_sums_kernel(const float* __restrict_
     }
 }
 
-// The fixed-order sum of reduce_kernel (mpr_aux.cu), one block per sweep.
+// The sum of a sweep's n partials in a fixed order, one block per sweep: thread t adds partials t, t + 256,
+// ..., then a tree (block_energy of the batched kernels adds in the same order).
 template <typename E>
 __global__ void __launch_bounds__(256) sweep_sums_kernel(const E* __restrict__ part, int n,
                                                          double* __restrict__ out)

@@ -63,7 +63,7 @@ inline bool too_large(cudaError_t e)
     return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
            e == cudaErrorLaunchOutOfResources;
 }
-// out[k] = the fixed-order sum of the n partials of sweep k (reduce_kernel's order), a block per sweep.
+// out[k] = the fixed-order sum of the n partials of sweep k, a block per sweep.
 cudaError_t launch_sums(const void* part, int n, int nsweeps, bool e32, double* out, cudaStream_t st);
 // The raw bond sums of nsweeps measured sweeps from their row sums, in the summation order of the
 // tile kernel and its reduction (bit-identical energies): out[k] for sweep k. part: nsweeps x
