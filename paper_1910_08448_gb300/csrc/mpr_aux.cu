@@ -289,7 +289,8 @@ __global__ void __launch_bounds__(kThreads) energy_final(const double* __restric
 // site (and one rounding less than dividing by n and by 2*pi at every site, which took about 20
 // instructions of the FP64 unit: 593 us at 4096^2, 9.4 ms at 16384^2). A block covers 256 columns
 // x kPredRows rows, all of a thread's loads in flight before K is ready; what is left is memory
-// traffic.
+// traffic. With a range near the smallest FP64 numbers K would lose bits or vanish: 2^200 K then, and sums
+// times 2^-200 (both exact).
 // --------------------------------------------------------------------------------------------
 constexpr int kPredRows = 8;
 
@@ -305,8 +306,9 @@ __global__ void __launch_bounds__(kThreads) predict_kernel(Layout L, const doubl
                                                            int nsamples, double* __restrict__ out)
 {
     __shared__ double s_k;
-    const double lo = range[0];
-    if (threadIdx.x == 0) s_k = (range[1] - lo) / (kTwoPi * (double)nsamples);
+    const double lo = range[0], width = range[1] - lo;
+    const bool tiny = width < 0x1p-900;
+    if (threadIdx.x == 0) s_k = (tiny ? width * 0x1p200 : width) / (kTwoPi * (double)nsamples);
     const int x = blockIdx.x * kThreads + threadIdx.x;
     bool first = true;
     for (long long y0 = (long long)blockIdx.y * kPredRows; y0 < L.Ly;
@@ -336,6 +338,7 @@ __global__ void __launch_bounds__(kThreads) predict_kernel(Layout L, const doubl
         for (int i = 0; i < kPredRows; ++i) {
             const int y = (int)y0 + i;
             if (x >= L.Lx || y >= L.Ly) continue;
+            if (tiny && !meas[i]) v[i] *= 0x1p-200;
             out[(size_t)y * L.Lx + x] = meas[i] ? v[i] : fma(v[i], k, lo);
         }
     }
