@@ -289,7 +289,8 @@ __global__ void __launch_bounds__(kThreads) energy_final(const double* __restric
 // site (and one rounding less than dividing by n and by 2*pi at every site, which took about 20
 // instructions of the FP64 unit: 593 us at 4096^2, 9.4 ms at 16384^2). A block covers 256 columns
 // x kPredRows rows, all of a thread's loads in flight before K is ready; what is left is memory
-// traffic. With a range near the smallest FP64 numbers K would lose bits or vanish: 2^200 K then, and sums
+// traffic. On grids of at most 128 columns it covers 2^lw >= Lx columns and as many more rows, its rows
+// interleaved over the threads (2 x 1000000: 256 columns a block leave 254 of 256 threads idle). With a range near the smallest FP64 numbers K would lose bits or vanish: 2^200 K then, and sums
 // times 2^-200 (both exact).
 // --------------------------------------------------------------------------------------------
 constexpr int kPredRows = 8;
@@ -303,21 +304,23 @@ __global__ void __launch_bounds__(kThreads) predict_kernel(Layout L, const doubl
                                                            const float* __restrict__ lo0,
                                                            const float* __restrict__ hi1,
                                                            const float* __restrict__ lo1,
-                                                           int nsamples, double* __restrict__ out)
+                                                           int nsamples, int lw, double* __restrict__ out)
 {
     __shared__ double s_k;
     const double lo = range[0], width = range[1] - lo;
     const bool tiny = width < 0x1p-900;
     if (threadIdx.x == 0) s_k = (tiny ? width * 0x1p200 : width) / (kTwoPi * (double)nsamples);
-    const int x = blockIdx.x * kThreads + threadIdx.x;
+    const int x = (blockIdx.x << lw) + (threadIdx.x & ((1 << lw) - 1));
+    const int ystep = kThreads >> lw;                // rows of the block side by side
+    const long long rows = (long long)kPredRows * ystep;
     bool first = true;
-    for (long long y0 = (long long)blockIdx.y * kPredRows; y0 < L.Ly;
-         y0 += (long long)gridDim.y * kPredRows) {   // rows beyond the 65535 grid limit
+    for (long long yb = blockIdx.y * rows; yb < L.Ly; yb += gridDim.y * rows) {   // (grid limit 65535)
+        const int y0 = (int)yb + (int)(threadIdx.x >> lw);
         double v[kPredRows];
         bool meas[kPredRows];
 #pragma unroll
         for (int i = 0; i < kPredRows; ++i) {
-            const int y = (int)y0 + i;
+            const int y = y0 + i * ystep;
             meas[i] = false;
             if (x >= L.Lx || y >= L.Ly) continue;
             const size_t s = (size_t)y * L.Lx + x;
@@ -336,7 +339,7 @@ __global__ void __launch_bounds__(kThreads) predict_kernel(Layout L, const doubl
         const double k = s_k;
 #pragma unroll
         for (int i = 0; i < kPredRows; ++i) {
-            const int y = (int)y0 + i;
+            const int y = y0 + i * ystep;
             if (x >= L.Lx || y >= L.Ly) continue;
             if (tiny && !meas[i]) v[i] *= 0x1p-200;
             out[(size_t)y * L.Lx + x] = meas[i] ? v[i] : fma(v[i], k, lo);
@@ -500,10 +503,13 @@ cudaError_t launch_predict(const Layout& L, const Precision&, const double* z,
                            const float* hi1, const float* lo1, int nsamples, double* out,
                            cudaStream_t st)
 {
-    const int ny = (L.Ly + kPredRows - 1) / kPredRows;
-    const dim3 grid(grid_for(L.Lx), ny < 65535 ? ny : 65535);
+    int lw = 8;
+    if (L.Lx <= 128)
+        for (lw = 1; 1 << lw < L.Lx;) ++lw;
+    const long long rows = (long long)kPredRows * (kThreads >> lw), ny = (L.Ly + rows - 1) / rows;
+    const dim3 grid((L.Lx + (1 << lw) - 1) >> lw, (unsigned)(ny < 65535 ? ny : 65535));
     predict_kernel<<<grid, kThreads, 0, st>>>(L, z, mask, range, acc0, acc1, hi0, lo0, hi1, lo1,
-                                              nsamples, out);
+                                              nsamples, lw, out);
     return cudaGetLastError();
 }
 

@@ -43,7 +43,7 @@ def _check(mpr, z, mask, setup, acc, n):
     # compensated in FP32 (2^-22.9 of the sum: two roundings of the last terms)
     scale = float(hi - lo)
     tol = scale * (2.0**-51 + n * 2.0**-52 if acc == "f64" else 2.0**-22) + max(abs(lo), abs(hi)) * 2.0**-52
-    assert np.abs((got - want)[free].astype(np.float64)).max() <= max(tol, 5e-324)
+    assert np.abs((got - want)[free].astype(np.float64)).max(initial=0.0) <= max(tol, 5e-324)
 
 
 @pytest.mark.parametrize("unit", [1.0, 1e-300, 3e-307, 1e-310, 5e-324, 1e300])
@@ -54,3 +54,13 @@ def test_any_range(mpr, unit, setup, acc):
     mask = (rng.random((40, 33)) < 0.4).astype(np.uint8)
     mask[0, :2] = 1
     _check(mpr, z, mask, setup, acc, 3)
+
+
+# widths around the powers of two that a block's columns are rounded to; heights around its rows
+@pytest.mark.parametrize("Lx", [2, 3, 4, 5, 31, 33, 64, 65, 128, 129, 257])
+@pytest.mark.parametrize("Ly", [2, 9, 1030])
+def test_any_shape(mpr, Lx, Ly):
+    rng = np.random.default_rng(2)
+    z, mask = rng.normal(50, 10, (Ly, Lx)), (rng.random((Ly, Lx)) < 0.4).astype(np.uint8)
+    mask[0, :2] = 1
+    _check(mpr, z, mask, "SDS", "f64", 2)
