@@ -203,10 +203,13 @@ __global__ void __launch_bounds__(kThreads) sample_energy_final(const double* __
 // of their black site: red neighbours of the row by shuffle, those above and below from the red
 // rows the warp keeps. A row with an angle outside [0, 7.5) (a state set by the caller) takes FP64.
 // 4096^2, FP16 spins: 2305 us with five FP64 sincos per black site.
-template <typename S>
+// NARROW (at most 14 half-lattice columns): a warp walks 32 / w strips side by side, w = 2^lw >= Lxh + 2 lanes
+// each; rows is even there, so that every strip is at a row of the same parity (2 x 1000000: 741 us with
+// a strip per warp).
+template <typename S, bool NARROW>
 __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __restrict__ red,
                                                           const S* __restrict__ black, double q,
-                                                          int64_t k65, int rows,
+                                                          int64_t k65, int rows, int lw,
                                                           double* __restrict__ part)
 {
     using V = typename std::conditional<sizeof(S) == 8, double, float>::type;
@@ -214,15 +217,17 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
     fixed::load_dirs(&energy::g_dirs, tab, threadIdx.x, kThreads);
     __syncthreads();
     const fixed::Split k = fixed::split(k65);
-    const int lane = threadIdx.x & 31;
-    const int nsx = (L.Lxh + 29) / 30;
+    const int w = NARROW ? 1 << lw : 32, side = NARROW ? 32 >> lw : 1;
+    const int lane = threadIdx.x & (w - 1);
+    const int nsx = NARROW ? 1 : (L.Lxh + 29) / 30;
     const long long nstrips = (long long)nsx * ((L.Ly + rows - 1) / rows);
     energy::Sum sum{0.0, 0.0};
-    for (long long st = (long long)blockIdx.x * energy::kWarpsPerBlock + (threadIdx.x >> 5);
-         st < nstrips; st += (long long)gridDim.x * energy::kWarpsPerBlock) {
-        const int sy = (int)(st / nsx), sx = (int)(st - (long long)sy * nsx);
+    for (long long st = ((long long)blockIdx.x * energy::kWarpsPerBlock + (threadIdx.x >> 5)) * side;
+         st < nstrips; st += (long long)gridDim.x * energy::kWarpsPerBlock * side) {
+        const int sy = NARROW ? (int)st + ((threadIdx.x & 31) >> lw) : (int)(st / nsx);
+        const int sx = NARROW ? 0 : (int)(st - (long long)sy * nsx);
         const int j = sx * 30 + lane - 1, y0 = sy * rows;
-        const int y1 = y0 + rows < L.Ly ? y0 + rows : L.Ly;
+        const int y1 = NARROW || y0 + rows < L.Ly ? y0 + rows : L.Ly;
         // a red angle at column j of row y (0 where there is none)
         auto is_red = [&](int y) { return j >= 0 && y >= 0 && y < L.Ly && 2 * j + (y & 1) < L.Lx; };
         auto red_at = [&](int y) -> V {
@@ -241,7 +246,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
             const energy::Vec ud = unit_at(y + 1, fd);
             const int o = (y + 1) & 1;   // black: x = 2j + o, red neighbours at columns j+o-1, j+o
             const int x = 2 * j + o;
-            const bool has = lane >= 1 && lane <= 30 && j < L.Lxh && x < L.Lx;
+            const bool has = lane >= 1 && lane <= w - 2 && j < L.Lxh && x < L.Lx && (!NARROW || y < L.Ly);
             const V fb = has ? load_as<V>(black[(size_t)y * L.pitch + j]) : (V)0;
             const bool ok = okd && okm && oku && fixed::in_range(fb);
             if (__all_sync(0xffffffffu, ok)) {
@@ -472,14 +477,23 @@ cudaError_t launch_sample_energy(const Layout& L, const double* z, const unsigne
     return cudaGetLastError();
 }
 
-// Strips of the energy kernel: 30 half-lattice columns x energy_rows rows.
-static int energy_rows(const Layout& L) { return energy::strip_rows((L.Lxh + 29) / 30, L.Ly); }
+// Strips of the energy kernel: 2^lw lanes (two of them neighbours' columns) x rows rows.
+struct EnergyStrips {
+    int lw = 5, rows;
+    long long warps;   // of 32 / 2^lw strips
+    explicit EnergyStrips(const Layout& L)
+    {
+        while (lw > 2 && (1 << (lw - 1)) >= L.Lxh + 2) --lw;
+        const int nsx = (L.Lxh + 29) / 30, side = 32 >> lw;
+        rows = energy::strip_rows(nsx, (L.Ly + side - 1) / side);
+        if (lw < 5) rows += rows & 1;
+        warps = ((long long)nsx * ((L.Ly + rows - 1) / rows) + side - 1) / side;
+    }
+};
 
 int energy_blocks(const Layout& L)
 {
-    const int rows = energy_rows(L);
-    const long long strips = (long long)((L.Lxh + 29) / 30) * ((L.Ly + rows - 1) / rows);
-    const long long b = (strips + energy::kWarpsPerBlock - 1) / energy::kWarpsPerBlock;
+    const long long b = (EnergyStrips(L).warps + energy::kWarpsPerBlock - 1) / energy::kWarpsPerBlock;
     return (int)(b < 152 * 6 ? b : 152 * 6);
 }
 
@@ -489,9 +503,10 @@ cudaError_t launch_energy_fp64(const Layout& L, const Precision& p, const void* 
 {
     return dispatch_store(p.store, [&](auto tag) {
         using S = decltype(tag);
-        energy_kernel<S><<<nblk, kThreads, 0, st>>>(L, static_cast<const S*>(ang0),
-                                                    static_cast<const S*>(ang1), q,
-                                                    fixed::turn_factor(q), energy_rows(L), part);
+        const EnergyStrips es(L);
+        auto* const kern = es.lw < 5 ? energy_kernel<S, true> : energy_kernel<S, false>;
+        kern<<<nblk, kThreads, 0, st>>>(L, static_cast<const S*>(ang0), static_cast<const S*>(ang1), q,
+                                        fixed::turn_factor(q), es.rows, es.lw, part);
         energy_final<<<1, kThreads, 0, st>>>(part, nblk, out);
         return cudaGetLastError();
     });

@@ -63,3 +63,27 @@ def test_state_energies_are_rounded_twice(mpr, Lx, Ly, q):
         _within(np.array(e).astype(LD) - _exact(np.array(states), q))
     finally:
         mpr.mpr_destroy(h)
+
+
+# a few columns, where a warp walks several strips side by side: widths around each strip width, last strips of
+# every height, angles outside the fixed range in some strips
+@pytest.mark.parametrize("Lx", [2, 3, 4, 5, 11, 12, 13, 27, 28, 29])
+@pytest.mark.parametrize("Ly", [2, 7, 33, 30011])
+@pytest.mark.parametrize("setup,far", [("DDD", False), ("HDS", False), ("DDD", True)])
+def test_state_energies_of_narrow_grids(mpr, Lx, Ly, setup, far):
+    rng = np.random.default_rng(42)
+    phi = rng.random((Ly, Lx)) * 2 * math.pi
+    if far:
+        for _ in range(3):
+            phi[rng.integers(1, Ly), rng.integers(Lx)] = rng.choice([-3.0, 9.0, 7.5])
+    mask = np.zeros((Ly, Lx), dtype=np.uint8)
+    mask[0, :2] = 1
+    h = mpr.mpr_create(np.arange(Lx)[None, :] + np.zeros((Ly, Lx)), mask)
+    try:
+        mpr.mpr_set_options(h, setup)
+        mpr.mpr_set_state(h, phi, 0)
+        err = LD(mpr.mpr_energy(h)[0]) - _exact(mpr.mpr_get_state(h)[0], 0.5)
+    finally:
+        mpr.mpr_destroy(h)
+    # out of range: five FP64 sincos and products per site, below 2^-50 each
+    assert abs(err) <= MOST + (2.0**-50 if far else 0.0)
