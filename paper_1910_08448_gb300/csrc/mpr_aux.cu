@@ -295,11 +295,14 @@ __global__ void __launch_bounds__(kThreads) energy_final(const double* __restric
 // instructions of the FP64 unit: 593 us at 4096^2, 9.4 ms at 16384^2). A block covers 256 columns
 // x kPredRows rows, all of a thread's loads in flight before K is ready; what is left is memory
 // traffic. On grids of at most 128 columns it covers 2^lw >= Lx columns and as many more rows, its rows
-// interleaved over the threads (2 x 1000000: 256 columns a block leave 254 of 256 threads idle). With a range near the smallest FP64 numbers K would lose bits or vanish: 2^200 K then, and sums
+// interleaved over the threads (2 x 1000000: 256 columns a block leave 254 of 256 threads idle).
+// Grids that would make fewer blocks than two per SM take one row per thread: there the FP64 unit's share
+// of a block is what the call waits for. With a range near the smallest FP64 numbers K would lose bits or vanish: 2^200 K then, and sums
 // times 2^-200 (both exact).
 // --------------------------------------------------------------------------------------------
 constexpr int kPredRows = 8;
 
+template <int ROWS>
 __global__ void __launch_bounds__(kThreads) predict_kernel(Layout L, const double* __restrict__ z,
                                                            const unsigned char* __restrict__ mask,
                                                            const double* __restrict__ range,
@@ -317,33 +320,43 @@ __global__ void __launch_bounds__(kThreads) predict_kernel(Layout L, const doubl
     if (threadIdx.x == 0) s_k = (tiny ? width * 0x1p200 : width) / (kTwoPi * (double)nsamples);
     const int x = (blockIdx.x << lw) + (threadIdx.x & ((1 << lw) - 1));
     const int ystep = kThreads >> lw;                // rows of the block side by side
-    const long long rows = (long long)kPredRows * ystep;
+    const long long rows = (long long)ROWS * ystep;
     bool first = true;
     for (long long yb = blockIdx.y * rows; yb < L.Ly; yb += gridDim.y * rows) {   // (grid limit 65535)
         const int y0 = (int)yb + (int)(threadIdx.x >> lw);
-        double v[kPredRows];
-        bool meas[kPredRows];
+        double v[ROWS];
+        bool meas[ROWS];
+        // every mask byte, then every value, without a branch on the mask between the rows: with one a
+        // thread's rows followed one another, 8 us longer at 64^2
 #pragma unroll
-        for (int i = 0; i < kPredRows; ++i) {
+        for (int i = 0; i < ROWS; ++i) {
             const int y = y0 + i * ystep;
-            meas[i] = false;
-            if (x >= L.Lx || y >= L.Ly) continue;
-            const size_t s = (size_t)y * L.Lx + x;
-            meas[i] = mask[s] != 0;
-            if (meas[i]) {
-                v[i] = z[s];
+            meas[i] = x < L.Lx && y < L.Ly && mask[(size_t)y * L.Lx + x] != 0;
+        }
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            const int y = y0 + i * ystep;
+            const bool there = x < L.Lx && y < L.Ly;
+            const size_t s = (size_t)y * L.Lx + x, idx = (size_t)y * L.pitch + (x >> 1);
+            const int c = (x + y) & 1;
+            if (acc0) {
+                const double* const p = meas[i] ? z + s : (c ? acc1 : acc0) + idx;
+                v[i] = there ? *p : 0.0;
             } else {
-                const size_t idx = (size_t)y * L.pitch + (x >> 1);
-                const int c = (x + y) & 1;
-                v[i] = acc0 ? (c ? acc1 : acc0)[idx]
-                            : (double)(c ? hi1 : hi0)[idx] - (double)(c ? lo1 : lo0)[idx];
+                // two words either way: of the value, or the sum and its compensation
+                const int* const zw = reinterpret_cast<const int*>(z + s);
+                const int* const p0 = meas[i] ? zw : reinterpret_cast<const int*>((c ? hi1 : hi0) + idx);
+                const int* const p1 = meas[i] ? zw + 1 : reinterpret_cast<const int*>((c ? lo1 : lo0) + idx);
+                const int w0 = there ? *p0 : 0, w1 = there ? *p1 : 0;
+                v[i] = meas[i] ? __hiloint2double(w1, w0)
+                               : (double)__int_as_float(w0) - (double)__int_as_float(w1);
             }
         }
         if (first) __syncthreads();   // s_k (every thread of the block makes the same trips)
         first = false;
         const double k = s_k;
 #pragma unroll
-        for (int i = 0; i < kPredRows; ++i) {
+        for (int i = 0; i < ROWS; ++i) {
             const int y = y0 + i * ystep;
             if (x >= L.Lx || y >= L.Ly) continue;
             if (tiny && !meas[i]) v[i] *= 0x1p-200;
@@ -521,10 +534,13 @@ cudaError_t launch_predict(const Layout& L, const Precision&, const double* z,
     int lw = 8;
     if (L.Lx <= 128)
         for (lw = 1; 1 << lw < L.Lx;) ++lw;
-    const long long rows = (long long)kPredRows * (kThreads >> lw), ny = (L.Ly + rows - 1) / rows;
-    const dim3 grid((L.Lx + (1 << lw) - 1) >> lw, (unsigned)(ny < 65535 ? ny : 65535));
-    predict_kernel<<<grid, kThreads, 0, st>>>(L, z, mask, range, acc0, acc1, hi0, lo0, hi1, lo1,
-                                              nsamples, lw, out);
+    const long long strips = (L.Ly + (kThreads >> lw) - 1) / (kThreads >> lw);   // rows of all threads
+    const unsigned nx = (unsigned)((L.Lx + (1 << lw) - 1) >> lw);
+    const bool few = strips * nx < (long long)kPredRows * 2 * 152;
+    const long long ny = few ? strips : (strips + kPredRows - 1) / kPredRows;
+    const dim3 grid(nx, (unsigned)(ny < 65535 ? ny : 65535));
+    auto* const kern = few ? predict_kernel<1> : predict_kernel<kPredRows>;
+    kern<<<grid, kThreads, 0, st>>>(L, z, mask, range, acc0, acc1, hi0, lo0, hi1, lo1, nsamples, lw, out);
     return cudaGetLastError();
 }
 

@@ -64,3 +64,12 @@ def test_any_shape(mpr, Lx, Ly):
     z, mask = rng.normal(50, 10, (Ly, Lx)), (rng.random((Ly, Lx)) < 0.4).astype(np.uint8)
     mask[0, :2] = 1
     _check(mpr, z, mask, "SDS", "f64", 2)
+
+
+# grids of many blocks, where a thread takes several rows (the sizes above take one): last blocks of few rows
+@pytest.mark.parametrize("Lx,Ly", [(2, 400007), (5, 100003), (64, 12001), (129, 2500), (257, 2003), (2003, 400)])
+@pytest.mark.parametrize("acc", ["f64", "kahan"])
+def test_several_rows_per_thread(mpr, Lx, Ly, acc):
+    rng = np.random.default_rng(3)
+    z, mask = rng.normal(50, 10, (Ly, Lx)), (rng.random((Ly, Lx)) < 0.4).astype(np.uint8)
+    _check(mpr, z, mask, "SDS", acc, 2)
