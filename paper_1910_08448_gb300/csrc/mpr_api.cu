@@ -392,11 +392,13 @@ mpr_status validate_options(const mpr_options* o)
 // - Up to four waves of four blocks: the T mod S tiles of the partial one when twice as many fit a
 //   wave (4096^2 HDS 28.4 / 27.7, 2560^2 SDS 14.5 / 13.3), else half of them (3000^2 HDS 17.2 / 16.6).
 // - Beyond that the partial wave is a small share (8192^2: 1 % slower with it).
+// - None in a single column of at most 32 half-columns, whose 32-column tiles have no halves (the 64-column
+//   code's instead: 28 x 50000 HDS 9.5 us per pass, 10.5 with them; 64 x 20000 bounded SDS 5.6 / 6.5).
 int split_tiles(const mpr_ctx* h, bool bounded)
 {
     const int per_sm = sweep_f32_plain_occupancy(h->prec, bounded), slots = per_sm * h->nsm;
     const int nt = sweep_f32_blocks(h->L);
-    if (slots <= 0 || nt >= 16 * h->nsm) return 0;
+    if (slots <= 0 || nt >= 16 * h->nsm || h->L.Lxh <= 32) return 0;
     if (nt <= slots) return (per_sm >= 4 && 10 * nt <= 9 * slots) || 2 * nt <= slots ? nt : 0;
     const int rem = nt % slots;
     return 2 * rem <= slots ? rem : rem / 2;

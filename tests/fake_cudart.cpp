@@ -37,13 +37,14 @@ void* get_memory(size_t n)
     return calloc(1, n ? n : 1);
 }
 
-cudaError_t launch(const void* f, void** args, size_t smem, bool programmatic, bool cooperative)
+cudaError_t launch(const void* f, unsigned grid, void** args, size_t smem, bool programmatic, bool cooperative)
 {
     Launch l;
     {
         std::lock_guard<std::mutex> lock(mu);
         l.name = names()[f];
     }
+    l.grid = grid;
     l.smem = smem;
     l.programmatic = programmatic;
     l.cooperative = cooperative;
@@ -113,9 +114,9 @@ cudaError_t __cudaPopCallConfiguration(dim3* grid, dim3* block, size_t* smem, vo
     *static_cast<void**>(st) = fake::pushed.stream;
     return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void** args, size_t smem, cudaStream_t)
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void** args, size_t smem, cudaStream_t)
 {
-    return fake::launch((const void*)k, args, smem, false, false);
+    return fake::launch((const void*)k, grid.x, args, smem, false, false);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args)
 {
@@ -125,11 +126,11 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
                c->attrs[i].val.programmaticStreamSerializationAllowed;
         coop |= c->attrs[i].id == cudaLaunchAttributeCooperative && c->attrs[i].val.cooperative;
     }
-    return fake::launch(f, args, c->dynamicSmemBytes, pdl, coop);
+    return fake::launch(f, c->gridDim.x, args, c->dynamicSmemBytes, pdl, coop);
 }
-cudaError_t cudaLaunchCooperativeKernel(const void* f, dim3, dim3, void** args, size_t smem, cudaStream_t)
+cudaError_t cudaLaunchCooperativeKernel(const void* f, dim3 grid, dim3, void** args, size_t smem, cudaStream_t)
 {
-    return fake::launch(f, args, smem, false, true);
+    return fake::launch(f, grid.x, args, smem, false, true);
 }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v)
 {

@@ -11,6 +11,7 @@ namespace fake {
 
 struct Launch {
     std::string name;      // mangled kernel name
+    unsigned grid;         // blocks along x
     size_t smem;           // dynamic shared memory
     bool programmatic;     // may start before the kernel in front of it has ended
     bool cooperative;

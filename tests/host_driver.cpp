@@ -33,7 +33,8 @@ void report(mpr_status s)
 {
     printf("status %d\n", (int)s);
     for (const fake::Launch& l : fake::launches)
-        printf("%s programmatic=%d cooperative=%d smem=%zu\n", l.name.c_str(), l.programmatic, l.cooperative, l.smem);
+        printf("%s programmatic=%d cooperative=%d grid=%u smem=%zu\n", l.name.c_str(), l.programmatic, l.cooperative,
+               l.grid, l.smem);
 }
 
 }  // namespace
@@ -42,8 +43,9 @@ int main(int argc, char** argv)
 {
     const char* const what = argc > 1 ? argv[1] : "";
     auto num = [&](int i) { return i < argc ? atoi(argv[i]) : 0; };
-    if (!strcmp(what, "run")) {   // Lx Ly equil samples
+    if (!strcmp(what, "run")) {   // Lx Ly equil samples [sweep kernel]
         mpr_handle h = handle(num(2), num(3));
+        if (argc > 6) mpr_set_sweep_kernel(h, num(6));
         fake::launches.clear();
         report(mpr_run(h, num(4), num(5)));
         mpr_destroy(h);

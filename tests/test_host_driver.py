@@ -99,3 +99,12 @@ def test_runs_without_memory_for_scratch(driver, shape, func):
     passes = [i for i, (n, _) in enumerate(calls) if _tile(n) or "12sweep_kernel" in n]
     assert len(sums) == 30 and all(len([p for p in passes if p < s]) % 2 == 0 for s in sums)
     assert len(passes) + 2 * sum(_resident(n) for n, _ in calls) * 5 == 2 * 35
+
+
+# a single column of at most 32 half-columns runs in 32-column tiles, which have no half-height form
+@pytest.mark.parametrize("shape", [(2, 40), (28, 50000), (64, 64), (64, 20000)])
+def test_narrow_grids_run_whole_tiles(driver, shape):
+    status, calls = driver("run", *shape, 3, 0, 0)
+    assert status == 0 and [a["grid"] for n, a in calls if _tile(n)] == 6 * [-(-shape[1] // 32)]
+    _, calls = driver("run", 66, shape[1], 3, 0, 0)
+    assert all(a["grid"] > -(-shape[1] // 32) for n, a in calls if _tile(n))   # a 64-column tile has halves
