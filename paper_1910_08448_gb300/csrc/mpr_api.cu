@@ -717,7 +717,7 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
         CHECK(harvest_profile(h));
         CU(cudaEventRecord(h->ev0, h->stream));
     }
-    if (h->rplan.nb > 0 && n >= 2 && h->sweep_force < 0 && !h->prop_on) {
+    if (h->rplan.nb > 0 && n >= h->rplan.least[flags & kMeasure ? 1 : 0] && h->sweep_force < 0 && !h->prop_on) {
         bool ran = true;
         CHECK(resident_sweeps(h, n, T, flags, &ran));
         if (ran) {

@@ -118,11 +118,20 @@ cudaError_t energies(const Layout& L, const float* er, int nsweeps, void* part, 
     return launch_sums(p, nt, nsweeps, sizeof(E) == 4, out, st);
 }
 
-}  // namespace
-
-Plan plan(const Layout& L, int store, int nsm)
+// A launch loads the lattice and stores it again; a run of two or three sweeps is worth that, except where the
+// tile kernel's passes are short: a single column of 32-column tiles. us per call of 2 and 3 plain sweeps,
+// resident / tile kernel: 64^2 25 / 21 and 25 / 24, 60 x 400 26 / 24 and 25 / 29, 60 x 20000 38 / 36 and 49 / 46 (2
+// and 3 measured ones 72 / 62, 85 / 82), but 256^2 25 / 30, 777 x 523 25 / 30, 1400 x 1200 38 / 42; and 12 x 100000
+// 50 / 90, whose tiles are mostly empty.
+void set_least(const Layout& L, int nsm, Plan* p)
 {
-    if (store == kF64 || nsm < 1) return Plan{};
+    if (p->nb == 0 || L.Lxh > 32) return;
+    if ((L.Ly + 31) / 32 <= nsm) p->least[0] = p->nb <= kCluster ? 4 : 3;
+    else if (p->pair && L.Lxh > 16) p->least[0] = p->least[1] = 4;
+}
+
+Plan any_plan(const Layout& L, int store, int nsm)
+{
     // Us per plain pass, SDS, measured. One cluster while its blocks stay short of warps: exchanges
     // cost 0.25 us there and 0.5 us through L2, but 16 blocks hold little (64^2 0.49 against 0.82;
     // 128^2 0.65 against 0.78; 140^2, 840 threads, 0.87 against 0.85, sampled 1.25 against 1.10).
@@ -139,6 +148,16 @@ Plan plan(const Layout& L, int store, int nsm)
     const Plan g2 = fine_plan(L, nsm, false, 2);
     if (g2.nb > 0) return g2;
     return coarse_plan(L, store, nsm);
+}
+
+}  // namespace
+
+Plan plan(const Layout& L, int store, int nsm)
+{
+    if (store == kF64 || nsm < 1) return Plan{};
+    Plan p = any_plan(L, store, nsm);
+    set_least(L, nsm, &p);
+    return p;
 }
 
 size_t halo_bytes(const Plan& p)

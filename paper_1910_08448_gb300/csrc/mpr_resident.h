@@ -22,6 +22,7 @@ struct Plan {
     int depth = 1;       // passes between two exchanges of boundary rows (fine_kernel: even)
     int G = 0;           // groups of four half-lattice columns in a row
     size_t smem = 0;     // dynamic shared memory of a block
+    int least[2] = {2, 2};   // fewest sweeps of a run that are worth the launch: plain, measured
 };
 
 struct Args {

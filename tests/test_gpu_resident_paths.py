@@ -54,7 +54,7 @@ def _problem(Lx, Ly, seed=61):
 def test_the_resident_kernel_runs(mpr, Lx, Ly, setup):
     h = _handle(mpr, _problem(Lx, Ly), setup)
     try:
-        assert _launches(mpr, h, 2, 0) == 1
+        assert _launches(mpr, h, 4, 0) == 1
         assert _launches(mpr, h, 37, 0) == 1
         assert _launches(mpr, h, 0, 3) == 3
         mpr.mpr_set_sweep_kernel(h, 0)
@@ -100,8 +100,26 @@ def test_one_sweep_behind_a_resident_launch(mpr, Lx, Ly, setup):
     for kind in (-1, 0):
         h = _handle(mpr, pr, setup, kind)
         try:
-            for equil in (2, 25, 3, 4097, 7):
+            for equil in (4, 25, 5, 4097, 7):
                 mpr.mpr_run(h, equil, 1)
+            out.append((mpr.mpr_get_state(h)[0], mpr.mpr_predict(h), mpr.mpr_get_info(h)["e_bond_mean"]))
+        finally:
+            mpr.mpr_destroy(h)
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    assert out[0][2] == out[1][2]
+
+
+# the shortest resident runs, two and three sweeps, on a cluster that exchanges rows every 4 passes and every 2, on
+# both grids, rows and row pairs
+@pytest.mark.parametrize("Lx,Ly", [(66, 64), (128, 127), (90, 767), (300, 300), (512, 401), (1400, 1200), (12, 60000)])
+@pytest.mark.parametrize("setup", ["SDS", "HDS"])
+def test_the_shortest_resident_runs(mpr, Lx, Ly, setup):
+    pr, out = _problem(Lx, Ly), []
+    for kind in (-1, 0):
+        h = _handle(mpr, pr, setup, kind)
+        try:
+            n = [_launches(mpr, h, *call) for call in ((2, 0), (3, 0), (0, 2), (0, 3))]
+            assert n == ([1, 1, 3, 3] if kind else [4, 6, 5, 7])
             out.append((mpr.mpr_get_state(h)[0], mpr.mpr_predict(h), mpr.mpr_get_info(h)["e_bond_mean"]))
         finally:
             mpr.mpr_destroy(h)

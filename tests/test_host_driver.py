@@ -79,7 +79,7 @@ def test_only_a_launch_that_is_too_large_falls_back(driver, shape):
 # front, and the resident kernel wrote both colours
 @pytest.mark.parametrize("shape", [(64, 64), (300, 300), (777, 523), (1400, 1200)])
 def test_a_pass_behind_a_resident_launch_is_no_programmatic_dependent(driver, shape):
-    for call in (("run", *shape, 2, 1), ("run", *shape, 25, 1), ("run", *shape, 4097, 1), ("tune", *shape, 3, 1)):
+    for call in (("run", *shape, 4, 1), ("run", *shape, 25, 1), ("run", *shape, 4097, 1), ("tune", *shape, 5, 1)):
         status, calls = driver(*call)
         behind = [i for i in range(1, len(calls)) if _tile(calls[i][0]) and not _tile(calls[i - 1][0])]
         assert status in (0, 4) and behind and all(_resident(calls[i - 1][0]) for i in behind)
@@ -108,3 +108,16 @@ def test_narrow_grids_run_whole_tiles(driver, shape):
     assert status == 0 and [a["grid"] for n, a in calls if _tile(n)] == 6 * [-(-shape[1] // 32)]
     _, calls = driver("run", 66, shape[1], 3, 0, 0)
     assert all(a["grid"] > -(-shape[1] // 32) for n, a in calls if _tile(n))   # a 64-column tile has halves
+
+
+# shapes and the fewest plain and measured sweeps that run resident: a cluster in one column of narrow tiles, a
+# grid there, a tall one, others
+@pytest.mark.parametrize("shape,plain,measured", [((64, 64), 4, 2), ((3, 3), 4, 2), ((60, 400), 3, 2),
+                                                  ((60, 20000), 4, 4), ((12, 100000), 2, 2), ((128, 128), 2, 2),
+                                                  ((256, 256), 2, 2), ((777, 523), 2, 2), ((1400, 1200), 2, 2)])
+def test_short_runs_take_the_quicker_kernel(driver, shape, plain, measured):
+    for n in (1, 2, 3, 4, 5):
+        for least, call in ((plain, (n, 0)), (measured, (0, n))):
+            status, calls = driver("run", *shape, *call)
+            assert status == 0 and any(_resident(name) for name, _ in calls) == (n >= least)
+            assert any(_tile(name) for name, _ in calls) == (n < least)
