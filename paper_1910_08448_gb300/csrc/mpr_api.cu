@@ -17,6 +17,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <new>
 #include <string>
@@ -175,6 +176,7 @@ constexpr uint64_t kPoolKeepBytes = 8ull << 30;
 constexpr int kMaxDevices = 64;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {};
+std::atomic<int> g_in_flight[kMaxDevices];   // see InFlight
 
 cudaError_t handle_pool(int device, cudaMemPool_t* out)
 {
@@ -717,7 +719,8 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
         CHECK(harvest_profile(h));
         CU(cudaEventRecord(h->ev0, h->stream));
     }
-    if (h->rplan.nb > 0 && n >= h->rplan.least[flags & kMeasure ? 1 : 0] && h->sweep_force < 0 && !h->prop_on) {
+    if (h->rplan.nb > 0 && n >= h->rplan.least[flags & kMeasure ? 1 : 0] &&
+        InFlight::now(h->device) <= h->rplan.runs && h->sweep_force < 0 && !h->prop_on) {
         bool ran = true;
         CHECK(resident_sweeps(h, n, T, flags, &ran));
         if (ran) {
@@ -917,6 +920,7 @@ mpr_status mpr_tune_temperature(mpr_handle h, double* T_out)
 {
     NvtxRange r("mpr_tune_temperature");
     if (!h) return fail(MPR_ERR_INVALID_ARG, "handle is NULL");
+    const InFlight running(h->device);
     const mpr_tuning& t = h->tune;
     const double e_s = h->e_s;
     const double tol = t.rel_tol * fabs(e_s);
@@ -967,6 +971,7 @@ mpr_status mpr_tune_heating(mpr_handle h, double factor, double* T_out)
 {
     NvtxRange r("mpr_tune_heating");
     if (!h) return fail(MPR_ERR_INVALID_ARG, "handle is NULL");
+    const InFlight running(h->device);
     if (!(factor > 1.0) || !(factor <= 100.0))
         return fail(MPR_ERR_INVALID_ARG, "heating factor %g outside (1, 100]", factor);
     if (h->free_lattice) return fail(MPR_ERR_STATE, "the lattice has no measured data");
@@ -1042,7 +1047,10 @@ mpr_status mpr_energy_curve(int Lx, int Ly, const mpr_options* opt, const mpr_tu
     CHECK(create_common(Lx, Ly, nullptr, nullptr, false, nullptr, &h, true));
     mpr_status s = opt ? mpr_set_options(h, opt) : MPR_OK;
     if (s == MPR_OK && tuning) s = mpr_set_tuning(h, tuning);
-    for (int i = 0; i < n && s == MPR_OK; ++i) s = probe(h, T[i], &e_out[i]);
+    if (s == MPR_OK) {
+        const InFlight running(h->device);
+        for (int i = 0; i < n && s == MPR_OK; ++i) s = probe(h, T[i], &e_out[i]);
+    }
     std::string keep = g_err;
     mpr_destroy(h);
     g_err = keep;
@@ -1094,6 +1102,7 @@ mpr_status mpr_run(mpr_handle h, int equil, int samples)
 {
     NvtxRange r("mpr_run");
     if (!h) return fail(MPR_ERR_INVALID_ARG, "handle is NULL");
+    const InFlight running(h->device);
     if (equil < 0 || samples < 0) return fail(MPR_ERR_INVALID_ARG, "negative sweep count");
     if (!h->have_T) return fail(MPR_ERR_STATE, "no temperature: tune or set it first");
     CHECK(sweeps(h, equil, h->T, 0));
@@ -1116,6 +1125,7 @@ mpr_status mpr_run_auto(mpr_handle h, int chunk, int max_equil, int samples, int
 {
     NvtxRange r("mpr_run_auto");
     if (!h) return fail(MPR_ERR_INVALID_ARG, "handle is NULL");
+    const InFlight running(h->device);
     if (chunk < 2 || max_equil < 0 || samples < 0)
         return fail(MPR_ERR_INVALID_ARG, "chunk %d must be >= 2, sweep counts >= 0", chunk);
     if (!h->have_T) return fail(MPR_ERR_STATE, "no temperature: tune or set it first");
@@ -1338,5 +1348,15 @@ const char* mpr_status_string(mpr_status s)
 const char* mpr_last_error(void) { return g_err.c_str(); }
 
 }  // extern "C"
+
+mpr::InFlight::InFlight(int device) : device_(device >= 0 && device < kMaxDevices ? device : 0)
+{
+    g_in_flight[device_].fetch_add(1, std::memory_order_relaxed);
+}
+mpr::InFlight::~InFlight() { g_in_flight[device_].fetch_sub(1, std::memory_order_relaxed); }
+int mpr::InFlight::now(int device)
+{
+    return g_in_flight[device >= 0 && device < kMaxDevices ? device : 0].load(std::memory_order_relaxed);
+}
 
 void mpr::set_last_error(const char* msg) { g_err = msg; }

@@ -632,6 +632,7 @@ mpr_status mpr_batch_fill(mpr_batch b, const double* T, int equil, int samples, 
         for (int i = 0; i < b->n; ++i)
             if (!(T[i] > 0.0) || !isfinite(T[i]))
                 return bfail(MPR_ERR_INVALID_ARG, "problem %d: temperature %g must be > 0", i, T[i]);
+    const InFlight running(b->device);
     prepare_fill(b, T);
     for (int i = 0; i < b->n; ++i) {
         batch::Dyn& d = b->P[(size_t)i].d;

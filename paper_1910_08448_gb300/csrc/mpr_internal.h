@@ -141,6 +141,20 @@ cudaError_t launch_fold_partials(double* acc, int* part, size_t n, cudaStream_t 
 cudaError_t launch_adapt_width(double* width, unsigned long long* count, long long n_pred,
                                double target, cudaStream_t st);
 
+// Calls that are running sweeps on a device, of any handle or batch, for as long as the object lives: what
+// several of them do best differs from what one does (resident::Plan::runs). Results do not depend on it.
+class InFlight {
+public:
+    explicit InFlight(int device);
+    ~InFlight();
+    InFlight(const InFlight&) = delete;
+    InFlight& operator=(const InFlight&) = delete;
+    static int now(int device);
+
+private:
+    int device_;
+};
+
 // Sets the message returned by mpr_last_error() on the calling thread.
 void set_last_error(const char* msg);
 

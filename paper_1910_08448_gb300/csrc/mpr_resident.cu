@@ -130,6 +130,23 @@ void set_least(const Layout& L, int nsm, Plan* p)
     else if (p->pair && L.Lxh > 16) p->least[0] = p->least[1] = 4;
 }
 
+// A resident launch keeps its SMs until its last sweep, so launches of several handles take turns unless two of
+// them fit side by side, where passes of the tile kernel share the device. us per run of 200 + 20 sweeps with 1 / 2
+// / 3 / 4 / 8 handles on threads and streams of their own, resident and (tile kernel):
+//   256^2 471 266 261 250 252 (1381 838 605 489 356): two fit (fine_kernel 80 registers, coarse_kernel 120)
+//   400 x 300 589 532 552 538 549 (1403 830 605 496 364)
+//   777 x 523 883 823 829 830 830 (1679 1165 797 620 493), 1024^2 1262 1175 1190 1191 1197 (1881 1328 1002 950 916)
+//   1400 x 1200 2154 2101 2098 2090 2094 (2701 1649 1528 1486 1503)
+// Mostly empty tiles (at most 16 half-columns) never catch up.
+void set_runs(const Layout& L, int nsm, Plan* p)
+{
+    constexpr int kAny = 1 << 30;
+    if (p->nb == 0) return;
+    const int per_sm = p->threads <= (p->fine ? 352 : 256) && 2 * (p->smem + 1024) <= kMaxSmem ? 2 : 1;
+    const long long sites = (long long)L.Lx * L.Ly;
+    p->runs = 2 * p->nb <= per_sm * nsm || L.Lxh <= 16 ? kAny : p->fine ? 3 : sites <= 1100000 ? 2 : 1;
+}
+
 Plan any_plan(const Layout& L, int store, int nsm)
 {
     // Us per plain pass, SDS, measured. One cluster while its blocks stay short of warps: exchanges
@@ -157,6 +174,7 @@ Plan plan(const Layout& L, int store, int nsm)
     if (store == kF64 || nsm < 1) return Plan{};
     Plan p = any_plan(L, store, nsm);
     set_least(L, nsm, &p);
+    set_runs(L, nsm, &p);
     return p;
 }
 

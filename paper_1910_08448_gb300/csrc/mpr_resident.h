@@ -23,6 +23,7 @@ struct Plan {
     int G = 0;           // groups of four half-lattice columns in a row
     size_t smem = 0;     // dynamic shared memory of a block
     int least[2] = {2, 2};   // fewest sweeps of a run that are worth the launch: plain, measured
+    int runs = 1;        // runs in flight on the device, this one included, up to which it is the quicker kernel
 };
 
 struct Args {

@@ -5,6 +5,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <condition_variable>
+#include <mutex>
 #include <thread>
 
 #include "fake_cudart.h"
@@ -88,6 +90,42 @@ int main(int argc, char** argv)
         fake::on_launch = nullptr;
         mpr_destroy(h);
         mpr_destroy(g);
+    } else if (!strcmp(what, "busy")) {   // Lx Ly, number of other handles that are in a run meanwhile
+        mpr_handle h = handle(num(2), num(3));
+        std::vector<mpr_handle> others;
+        for (int i = 0; i < num(4); ++i) others.push_back(handle(40, 40));
+        std::vector<std::thread> ts;
+        std::mutex mu;
+        std::condition_variable cv;
+        int waiting = 0;
+        bool go = false;
+        const std::thread::id me = std::this_thread::get_id();
+        fake::on_launch = [&](const fake::Launch&) {   // the others stop at their first launch
+            if (std::this_thread::get_id() == me) return 0;
+            std::unique_lock<std::mutex> lock(mu);
+            ++waiting;
+            cv.notify_all();
+            cv.wait(lock, [&] { return go; });
+            return 0;
+        };
+        for (mpr_handle g : others) ts.emplace_back([g] { mpr_run(g, 1, 0); });
+        {
+            std::unique_lock<std::mutex> lock(mu);
+            cv.wait(lock, [&] { return waiting == (int)others.size(); });
+        }
+        fake::launches.clear();
+        report(mpr_run(h, 5, 4));
+        {
+            std::lock_guard<std::mutex> lock(mu);
+            go = true;
+        }
+        cv.notify_all();
+        for (std::thread& t : ts) t.join();
+        fake::on_launch = nullptr;
+        fake::launches.clear();
+        if (mpr_run(h, 5, 4) != MPR_OK || !is_resident(fake::launches.front())) return 1;   // alone again
+        for (mpr_handle g : others) mpr_destroy(g);
+        mpr_destroy(h);
     } else if (!strcmp(what, "refuse")) {   // Lx Ly, error code of the resident launches
         mpr_handle h = handle(num(2), num(3));
         fake::launches.clear();

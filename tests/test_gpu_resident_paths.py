@@ -63,7 +63,7 @@ def test_the_resident_kernel_runs(mpr, Lx, Ly, setup):
         mpr.mpr_destroy(h)
 
 
-@pytest.mark.parametrize("shapes", [((1400, 1200), (1024, 1024)), ((777, 523), (700, 400))])
+@pytest.mark.parametrize("shapes", [((1024, 1024), (900, 900)), ((777, 523), (700, 400))])
 def test_two_sizes_on_two_threads(mpr, shapes):
     """Short runs of two lattices of one resident kernel, of different shared memory."""
     import torch

@@ -121,3 +121,13 @@ def test_short_runs_take_the_quicker_kernel(driver, shape, plain, measured):
             status, calls = driver("run", *shape, *call)
             assert status == 0 and any(_resident(name) for name, _ in calls) == (n >= least)
             assert any(_tile(name) for name, _ in calls) == (n < least)
+
+
+# runs in flight (this one included) up to which a lattice runs resident
+@pytest.mark.parametrize("shape,most", [((64, 64), 9), ((200, 150), 9), ((256, 256), 9), ((400, 300), 3),
+                                        ((512, 400), 9), ((777, 523), 2), ((1024, 1024), 2), ((1400, 1200), 1),
+                                        ((12, 100000), 9)])
+def test_handles_that_run_at_once_share_the_device(driver, shape, most):
+    for others in range(9):
+        status, calls = driver("busy", *shape, others)
+        assert status == 0 and any(_resident(n) for n, _ in calls) == (others + 1 <= most)
