@@ -706,7 +706,12 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
     a.err = dev_err(h);
     a.wait_ns = 2000000000LL;   // 2 s: a TMA copy lands in microseconds
     a.stall_test = 0;
-    a.nsplit = h->prop_on ? h->nsplit_prop : h->nsplit;   // read by the plain-pass launches only
+    // read by the plain-pass launches only; none where the passes of other runs fill the device (us per run of 200
+    // + 20 sweeps, 4 at once, with / without: 1400 x 1200 1497 / 1428, 2501 x 1333 BDS 2730 / 2497, but 777 x 523
+    // 642 / 807)
+    const int runs = InFlight::now(h->device);
+    const bool full = runs > 1 && (long long)runs * sweep_f32_blocks(h->L) > 4LL * h->nsm;
+    a.nsplit = full ? 0 : h->prop_on ? h->nsplit_prop : h->nsplit;
     a.late = h->late;   // read by the plain-pass launches only (the red pass of a measured sweep too)
     // bounded proposals; the width adapts after every sweep that does not sample
     const bool adapt = h->prop_on && h->prop_target > 0.0 && !(flags & kSample);

@@ -131,3 +131,13 @@ def test_handles_that_run_at_once_share_the_device(driver, shape, most):
     for others in range(9):
         status, calls = driver("busy", *shape, others)
         assert status == 0 and any(_resident(n) for n, _ in calls) == (others + 1 <= most)
+
+
+# half-height tiles shorten the last wave of a pass that has the device to itself
+@pytest.mark.parametrize("shape,most", [((777, 523), 8), ((1400, 1200), 2), ((2000, 1500), 1)])
+def test_no_half_height_tiles_where_other_runs_fill_the_device(driver, shape, most):
+    tiles = -(-((shape[0] + 1) // 2) // 128) * -(-shape[1] // 32)
+    for others in range(9):
+        _, calls = driver("busy", *shape, others)
+        plain = [a["grid"] for n, a in calls if _tile(n)][:10]
+        assert len(plain) in (0, 10) and all((g > tiles) == (others + 1 <= most) for g in plain)
