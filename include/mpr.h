@@ -222,12 +222,17 @@ mpr_status mpr_set_proposal(mpr_handle h, double width, double target);
 /* Current half-width of the bounded proposal (0 when proposals are uniform); synchronises. */
 mpr_status mpr_get_proposal(mpr_handle h, double* width);
 
-/* Test hook for the bounded wait of the TMA kernel: in the next pass that runs with kind 1, block
- * 0 issues no copy for its first tile, so its mbarrier wait runs out after timeout_s (0 < timeout_s
- * <= 10); the block records MPR_ERR_DEVICE_TIMEOUT and returns, the other blocks finish, nothing
- * faults or hangs, and the call that synchronises next (e.g. mpr_run) returns
- * MPR_ERR_DEVICE_TIMEOUT. That pass leaves the tiles of block 0 unchanged (the chain deviates);
- * the handle stays usable. INVALID_ARG if the handle cannot run kind 1. */
+/* Test hook for the bounded waits, of the next launch that has any, for timeout_s (0 < timeout_s <= 10):
+ *   - a pass with kind 1: block 0 issues no copy for its first tile, so its mbarrier wait runs out; it records
+ *     MPR_ERR_DEVICE_TIMEOUT and returns, the other blocks finish. Its tiles stay as they were;
+ *   - a resident launch of several bands (see mpr_set_sweep_kernel; plain sweeps of FP32 spins at q = 1/2 only):
+ *     the first band sends none of its rows, so the wait of the band beside it runs out; that band records the error, the others see it at their next
+ *     wait, and all of them leave, each after the sweeps it had done.
+ * Nothing faults or hangs, and the call that synchronises next (e.g. mpr_run) returns
+ * MPR_ERR_DEVICE_TIMEOUT. The sweep counter counts the whole run, the angles are those of a chain that
+ * was cut off (prediction sites stay in [0, 2 pi]), and the samples and energies of the run are undefined:
+ * a caller starts over from mpr_set_options, or from a saved state. The handle stays usable.
+ * INVALID_ARG if the handle cannot run kind 1. */
 mpr_status mpr_inject_tma_stall(mpr_handle h, double timeout_s);
 
 /* State access for checkpoints and tests: angles as Lx*Ly doubles, row-major, host memory.

@@ -133,7 +133,7 @@ struct mpr_ctx {
     TmaMaps tma{};
     int nsm = 0;                         // SMs of the device
     int sweep_force = -1;                // mpr_set_sweep_kernel: -1 automatic, 0, 1
-    long long stall_ns = 0;              // mpr_inject_tma_stall: wait limit of the next TMA pass
+    long long stall_ns = 0;              // mpr_inject_tma_stall: wait limit of the next launch that waits
     int sweep_kind = -1;                 // automatic choice (-1 until made)
     int nsplit = 0, nsplit_prop = 0;     // plain passes of the tile kernel: last tiles split in two
                                          // (uniform, bounded proposals)
@@ -640,7 +640,6 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
     a.nl2eTf = -1.4426950408889634f * (float)(1.0 / T);
     a.keys = philox_sched(0u, 0u, kTagMetropolis, 0u, a.seed_lo, a.seed_hi);
     a.err = dev_err(h);
-    a.wait_ns = 2000000000LL;
     // FP64 sums take each sample directly (with FP16 spins too: every add is exact, so the sums are
     // the bits of the fixed-point partials')
     const int sample = (flags & kSample) ? (h->prec.acc == 0 ? 1 : 2) : 0;
@@ -654,8 +653,12 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
         a.sweep = h->sweep;
         a.depth = p.fine ? std::min(p.depth, 2 * (m - 1)) : 1;
         a.epoch = p.cluster ? 0u : h->epoch;
-        const cudaError_t e = resident::launch(p, h->prec.store, measure, sample, a.qf == 0.5f, a,
-                                               h->stream);
+        // injected stall: this launch only
+        const bool stall = h->stall_ns > 0 && p.nb > 1 && !measure && h->prec.store == kF32 && a.qf == 0.5f;
+        a.wait_ns = stall ? h->stall_ns : 2000000000LL;   // 2 s: a neighbour's rows come within microseconds
+        const cudaError_t e =
+            stall ? resident::launch_stalled(p, a, h->stream)
+                  : resident::launch(p, h->prec.store, measure, sample, a.qf == 0.5f, a, h->stream);
         if (resident::too_large(e) && k == 0) {
             cudaGetLastError();
             h->rplan.nb = 0;
@@ -663,6 +666,7 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
             return MPR_OK;
         }
         CU(e);
+        if (stall) h->stall_ns = 0;
         h->after_resident = true;
         if (measure)
             CU(resident::launch_energies(h->L, h->prec.energy == 1, h->er, m, h->rpart,

@@ -175,7 +175,9 @@ __device__ __forceinline__ float4 unit_uniforms(const uint4& w0, const uint4& w1
     }
 }
 
-template <typename S, bool MEASURE, int SAMPLE, int QM, bool CLUSTER>
+// STALL: test hook, the first band sends nothing (kernels of their own: the condition alone cost the others 3 %
+// at 64^2).
+template <typename S, bool MEASURE, int SAMPLE, int QM, bool CLUSTER, bool STALL = false>
 __global__ void __launch_bounds__(kFineThreads, 1) fine_kernel(const __grid_constant__ Args A)
 {
     extern __shared__ __align__(16) unsigned char dsm[];
@@ -263,7 +265,7 @@ __global__ void __launch_bounds__(kFineThreads, 1) fine_kernel(const __grid_cons
     }
     // boundary rows: where this unit's words go and come from (of the colour moved last; row
     // dist - 1, the other colour K - 1 rows further)
-    const bool up = mine && above < K && b > 0, down = mine && below < K && b + 1 < nb;
+    const bool up = mine && above < K && b > 0, down = mine && below < K && b + 1 < nb && !(STALL && b == 0);
     unsigned long long* const to_up = slot<CLUSTER>(A, mail, nb, up ? b - 1 : b, 1, up ? above : 0) + jc;
     unsigned long long* const to_down = slot<CLUSTER>(A, mail, nb, down ? b + 1 : b, 0, down ? below : 0) + jc;
     const bool take = unit && dist > 0;
@@ -488,7 +490,7 @@ struct QuadRow {
     }
 };
 
-template <typename S, bool MEASURE, int SAMPLE, int QM, bool PAIR>
+template <typename S, bool MEASURE, int SAMPLE, int QM, bool PAIR, bool STALL = false>
 __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_kernel(const __grid_constant__ Args A)
 {
     extern __shared__ __align__(16) unsigned char dsm[];
@@ -602,7 +604,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_kernel(const __grid_
                         put2(p + 2, tagged(m.fn[1].x, tag + 1u), tagged(m.fn[1].y, tag + 1u));
                     };
                     if (!last && i == 0 && b > 0) send(b - 1, 1);
-                    if (!last && i == nr - 1 && b + 1 < nb) send(b + 1, 0);
+                    if (!last && i == nr - 1 && b + 1 < nb && !(STALL && b == 0)) send(b + 1, 0);
                     Pack4<S> pk;
 #pragma unroll
                     for (int t = 0; t < 2; ++t) {
@@ -651,13 +653,13 @@ out:
     }
 }
 
-template <typename S, bool MEASURE, int SAMPLE, int QM>
+template <typename S, bool MEASURE, int SAMPLE, int QM, bool STALL = false>
 cudaError_t go_shape(const Plan& p, const Args& a, cudaStream_t st)
 {
-    void (*kern)(const Args) = p.cluster ? fine_kernel<S, MEASURE, SAMPLE, QM, true>
-                               : p.fine  ? fine_kernel<S, MEASURE, SAMPLE, QM, false>
-                               : p.pair  ? coarse_kernel<S, MEASURE, SAMPLE, QM, true>
-                                         : coarse_kernel<S, MEASURE, SAMPLE, QM, false>;
+    void (*kern)(const Args) = p.cluster ? fine_kernel<S, MEASURE, SAMPLE, QM, true, STALL>
+                               : p.fine  ? fine_kernel<S, MEASURE, SAMPLE, QM, false, STALL>
+                               : p.pair  ? coarse_kernel<S, MEASURE, SAMPLE, QM, true, STALL>
+                                         : coarse_kernel<S, MEASURE, SAMPLE, QM, false, STALL>;
     // An attribute belongs to the function, and handles of other host threads launch it too: always the same
     // value, the most a plan takes. (With p.smem here, a smaller lattice's value that landed between
     // a larger one's call and its launch made that launch fail.)

@@ -59,6 +59,8 @@ size_t halo_bytes(const Plan& p);
 // nsweeps hybrid sweeps; sample: 0 none, 1 FP64 sums, 2 Kahan sums (only with measure).
 cudaError_t launch(const Plan& p, int store, bool measure, int sample, bool qhalf, const Args& a,
                    cudaStream_t st);
+// Test hook: the same launch, plain, FP32 spins, q = 1/2, in which the first band sends nothing.
+cudaError_t launch_stalled(const Plan& p, const Args& a, cudaStream_t st);
 // The launch was refused because the device cannot hold its blocks at once (nothing ran).
 inline bool too_large(cudaError_t e)
 {

@@ -125,3 +125,34 @@ def test_the_shortest_resident_runs(mpr, Lx, Ly, setup):
             mpr.mpr_destroy(h)
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
     assert out[0][2] == out[1][2]
+
+
+# the first band withholds its rows: its neighbour's bounded wait runs out, every block leaves, the error is
+# reported once and the handle goes on (fine grid of 17 and of 150 bands, one row and row pairs per thread)
+@pytest.mark.parametrize("Lx,Ly", [(258, 34), (300, 300), (777, 523), (1024, 1024)])
+@pytest.mark.parametrize("call", [(40, 0), (7, 20)])
+def test_a_wait_that_runs_out_is_reported(mpr, Lx, Ly, call):
+    pr = _problem(Lx, Ly)
+    h = _handle(mpr, pr)
+    try:
+        want = []
+        for stall in (True, False):
+            mpr.mpr_set_options(h, "SDS", seed=31)
+            mpr.mpr_set_temperature(h, 0.2)
+            mpr.mpr_run(h, 4, 0)
+            if stall:
+                mpr.mpr_inject_tma_stall(h, 0.05)
+                with pytest.raises(mpr.MPRError) as e:
+                    mpr.mpr_run(h, *call)
+                assert e.value.status == mpr.MPR_ERR_DEVICE_TIMEOUT
+                state, sweep = mpr.mpr_get_state(h)
+                assert sweep == 4 + sum(call) and state.min() >= 0.0 and state.max() <= 6.2831855
+                mpr.mpr_set_options(h, "SDS", seed=31)
+                mpr.mpr_set_temperature(h, 0.2)
+                mpr.mpr_run(h, 4, 0)
+            mpr.mpr_run(h, 30, 20)   # tags of the run that was cut off are never taken for new ones
+            want.append((mpr.mpr_get_state(h)[0], mpr.mpr_predict(h), mpr.mpr_get_info(h)["e_bond_mean"]))
+        assert np.array_equal(want[0][0], want[1][0]) and np.array_equal(want[0][1], want[1][1])
+        assert want[0][2] == want[1][2]
+    finally:
+        mpr.mpr_destroy(h)
