@@ -703,7 +703,6 @@ mpr_status sweeps(mpr_ctx* h, int n, double T, int flags)
     a.problem = 0;
     a.q = h->opt.q;
     a.T = T;
-    a.invT = 1.0 / T;
     a.qf = (float)h->opt.q;
     a.invTf = (float)(1.0 / T);
     a.nl2eTf = -1.4426950408889634f * a.invTf;   // FP32 product, as the batched kernels form it

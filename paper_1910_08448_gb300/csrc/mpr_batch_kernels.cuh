@@ -258,7 +258,6 @@ __device__ __forceinline__ void tile_body(const Args* __restrict__ A, int t, int
     a.problem = (uint32_t)p;
     a.q = A->q;
     a.T = 0.0;
-    a.invT = 0.0;        // the FP32 tile uses qf and invTf only
     a.qf = A->qf;
     a.invTf = __ldcg(&P.d.invTf);
     a.nl2eTf = -1.4426950408889634f * a.invTf;

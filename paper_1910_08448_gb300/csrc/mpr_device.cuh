@@ -1,6 +1,5 @@
-// mpr_device.cuh -- device building blocks of the MPR sweeps: Philox-4x32-10, storage
-// conversions and the precision-dispatched math of the three precision axes of Sec. 2
-// (spins X_S, energy X_E, functions X_F).
+// mpr_device.cuh -- device building blocks of the MPR sweeps: Philox-4x32-10 and the conversions of
+// the spin storages X_S (Sec. 2).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -134,33 +133,5 @@ template <> __device__ __forceinline__ __half store_from<__half>(double v) { ret
 template <> __device__ __forceinline__ __half store_from<__half>(float v) { return __float2half_rn(v); }
 template <> __device__ __forceinline__ __nv_bfloat16 store_from<__nv_bfloat16>(double v) { return __double2bfloat16(v); }
 template <> __device__ __forceinline__ __nv_bfloat16 store_from<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
-
-// ---------------------------------------------------------------------------------------------
-// Function precision X_F: FP64 library functions, or the FP32 hardware intrinsics (Sec. 2: the
-// hardware-intrinsic versions are used for all SP function evaluations).
-// ---------------------------------------------------------------------------------------------
-template <typename F> struct Math;
-
-template <> struct Math<double> {
-    static __device__ __forceinline__ void sincos_(double a, double* s, double* c) { sincos(a, s, c); }
-    static __device__ __forceinline__ double exp_neg_over(double dE, double T, double /*invT*/) { return exp(-dE / T); }
-    static __device__ __forceinline__ double atan2_(double y, double x) { return atan2(y, x); }
-    static __device__ __forceinline__ double uniform(uint32_t w) { return uniform_d(w); }
-    static __device__ __forceinline__ double two_pi() { return kTwoPi; }
-    static __device__ __forceinline__ double floor_(double v) { return floor(v); }
-};
-
-template <> struct Math<float> {
-    static __device__ __forceinline__ void sincos_(float a, float* s, float* c) { __sincosf(a, s, c); }
-    static __device__ __forceinline__ float exp_neg_over(float dE, float /*T*/, float invT) { return __expf(-dE * invT); }
-    static __device__ __forceinline__ float atan2_(float y, float x) { return atan2f(y, x); }
-    static __device__ __forceinline__ float uniform(uint32_t w) { return uniform_f(w); }
-    static __device__ __forceinline__ float two_pi() { return kTwoPiF; }
-    static __device__ __forceinline__ float floor_(float v) { return floorf(v); }
-};
-
-template <typename F> struct Vec2;
-template <> struct Vec2<double> { using type = double2; };
-template <> struct Vec2<float> { using type = float2; };
 
 }  // namespace mpr

@@ -250,10 +250,11 @@ MPR_HD double to_double_q60(uint64_t v)
 }
 
 // Twice the argument of (hx, hy) in turns, given t0 = that argument modulo pi as a fraction of a
-// turn with 32 bits, known to about 1e-6 rad. hx, hy with 60 fraction bits, at most 4 in size and
-// at least 2^-10 in one component. The vector is turned back by t0; what is left of it is
-// num / den = tan of the rest (its cube is below 2^-58). The quotient is an FP32 pair: 46 bits of
-// a rest below 2^-18.
+// turn with 32 bits. hx, hy with 60 fraction bits, at most 4 in size and at least 2^-10 in one
+// component. t0 comes from fields cut to 28 fraction bits and an FP32 arc tangent: off by 1.5e-6 rad, and by
+// 2^-27.5 / |h| more in small fields (5.4e-6 rad at 2^-10). The vector is turned back by t0; what is left of
+// it is num / den = tan of the rest, whose cube (2^-58 at |h| = 1, 2^-52 at 2^-10) lies below what the field's
+// own last bits do to the angle there (2^-58 / |h|). The quotient is an FP32 pair: 46 bits of the rest.
 MPR_HD uint64_t doubled_arg(const Dir* tab, int64_t hx, int64_t hy, int32_t t0)
 {
     int64_t c0, s0;

@@ -60,7 +60,7 @@ struct SweepArgs {
     int colour;
     int flags;
     uint32_t seed_lo, seed_hi, sweep, problem;
-    double q, T, invT;
+    double q, T;
     float qf, invTf;           // the same in FP32 for the FP32-function kernel (no FP64 on device)
     float nl2eTf;              // -log2(e) * invTf as one FP32 product: exp(-dE/T) = 2^(dE * nl2eTf)
     int* err;                  // device error word (MPR_ERR_DEVICE_TIMEOUT) or NULL

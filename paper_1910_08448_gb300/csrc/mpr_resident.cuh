@@ -118,8 +118,8 @@ struct Band {
 // Words of row `row` of the exchange with tag parity 0, in the slots of block `to`, side 0 (rows
 // above its band) or 1; parity 1 lies slot_stride further.
 template <bool CLUSTER>
-__device__ __forceinline__ unsigned long long* slot(const Args& A, unsigned long long* mail, int nb, int to,
-                                                    int side, int row)
+__device__ __forceinline__ unsigned long long* slot(const Args& A, unsigned long long* mail, int to, int side,
+                                                    int row)
 {
     const int RS = halo_rows(A.depth);
     if constexpr (CLUSTER)
@@ -266,11 +266,11 @@ __global__ void __launch_bounds__(kFineThreads, 1) fine_kernel(const __grid_cons
     // boundary rows: where this unit's words go and come from (of the colour moved last; row
     // dist - 1, the other colour K - 1 rows further)
     const bool up = mine && above < K && b > 0, down = mine && below < K && b + 1 < nb && !(STALL && b == 0);
-    unsigned long long* const to_up = slot<CLUSTER>(A, mail, nb, up ? b - 1 : b, 1, up ? above : 0) + jc;
-    unsigned long long* const to_down = slot<CLUSTER>(A, mail, nb, down ? b + 1 : b, 0, down ? below : 0) + jc;
+    unsigned long long* const to_up = slot<CLUSTER>(A, mail, up ? b - 1 : b, 1, up ? above : 0) + jc;
+    unsigned long long* const to_down = slot<CLUSTER>(A, mail, down ? b + 1 : b, 0, down ? below : 0) + jc;
     const bool take = unit && dist > 0;
     const unsigned long long* const from =
-        slot<CLUSTER>(A, mail, nb, b, above < 0 ? 0 : 1, take ? dist - 1 : 0) + jc;
+        slot<CLUSTER>(A, mail, b, above < 0 ? 0 : 1, take ? dist - 1 : 0) + jc;
     const size_t parity = slot_stride<CLUSTER>(A, nb), other = (size_t)(K - 1) * 4 * G;
     const int par = y & 1;   // role of the row: its parity for colour 0, the opposite for colour 1
     const float4* const uu = uni + 2 * ((y >> 1) - P0) * G + (jc >> 1);
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_kernel(const __grid_
                     // a neighbour's boundary row, these four columns: read by this thread only
                     auto take = [&](int side, int rr) {
                         const unsigned long long* const p =
-                            slot<false>(A, nullptr, nb, b, side, 0) + (tag & 1u) * parity + 4 * g;
+                            slot<false>(A, nullptr, b, side, 0) + (tag & 1u) * parity + 4 * g;
                         float x[4], vc[4], vs[4];
                         if (!wait2(A, p, tag, x[0], x[1]) || !wait2(A, p + 2, tag, x[2], x[3])) bad = true;
 #pragma unroll
@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) coarse_kernel(const __grid_
                     m.run(A, vb, vo, r, g, own(c, i, g), frozen(c, i, g), w0, w1, w2, q, width, inv_q);
                     auto send = [&](int to, int side) {
                         unsigned long long* const p =
-                            slot<false>(A, nullptr, nb, to, side, 0) + ((tag + 1u) & 1u) * parity + 4 * g;
+                            slot<false>(A, nullptr, to, side, 0) + ((tag + 1u) & 1u) * parity + 4 * g;
                         put2(p, tagged(m.fn[0].x, tag + 1u), tagged(m.fn[0].y, tag + 1u));
                         put2(p + 2, tagged(m.fn[1].x, tag + 1u), tagged(m.fn[1].y, tag + 1u));
                     };

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(256, 3) sweep_kernel(const __grid_constant__ S
                         inside = fp >= 0.0 && fp < kTwoPi;
                         tp = inside ? fixed::turns(fp, k65) : t0;
                     }
-                    // FP32 estimates: hx, hy to 2.4e-7 of their size, the sines and cosines to
+                    // FP32 estimates: hx, hy to 6e-8 of their size and 2^-28, the sines and cosines to
                     // 9e-7 (angle rounded to FP32 in [-pi, pi], intrinsics to 2^-21.2), so dE to
                     // 2e-6 (|hx| + |hy|) and its roundings; T |ln u| to 6e-7 of its size and
                     // 5e-7 T. Accepted iff dE < T |ln u| (which is >= 0).
