@@ -210,7 +210,7 @@ template <typename S, bool NARROW>
 __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __restrict__ red,
                                                           const S* __restrict__ black, double q,
                                                           int64_t k65, int rows, int lw,
-                                                          double* __restrict__ part)
+                                                          energy::Sum* __restrict__ part)
 {
     using V = typename std::conditional<sizeof(S) == 8, double, float>::type;
     __shared__ fixed::Dir tab[fixed::kDirs];
@@ -221,7 +221,8 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
     const int lane = threadIdx.x & (w - 1);
     const int nsx = NARROW ? 1 : (L.Lxh + 29) / 30;
     const long long nstrips = (long long)nsx * ((L.Ly + rows - 1) / rows);
-    energy::Sum sum{0.0, 0.0};
+    energy::Sum sum{0, 0};
+    bool nan = false;
     for (long long st = ((long long)blockIdx.x * energy::kWarpsPerBlock + (threadIdx.x >> 5)) * side;
          st < nstrips; st += (long long)gridDim.x * energy::kWarpsPerBlock * side) {
         const int sy = NARROW ? (int)st + ((threadIdx.x & 31) >> lw) : (int)(st / nsx);
@@ -266,7 +267,7 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
                     if (y > 0) { sincos(q * (double)fu, &sn, &cs); hx += cs; hy += sn; }
                     if (y + 1 < L.Ly) { sincos(q * (double)fd, &sn, &cs); hx += cs; hy += sn; }
                     sincos(q * (double)fb, &sn, &cs);
-                    sum.add_fp64(cs * hx + sn * hy);
+                    acc += energy::term_fp64(cs * hx + sn * hy, &nan);
                 }
             }
             fu = fm;
@@ -278,10 +279,10 @@ __global__ void __launch_bounds__(kThreads) energy_kernel(Layout L, const S* __r
         }
         sum.add(acc);
     }
-    energy::block_sum(sum, part);
+    energy::store_sum(sum, nan, part);
 }
 
-__global__ void __launch_bounds__(kThreads) energy_final(const double* __restrict__ part, int n,
+__global__ void __launch_bounds__(kThreads) energy_final(const energy::Sum* __restrict__ part, int n,
                                                          double* __restrict__ out)
 {
     const double s = energy::final_sum(part, n);
@@ -517,10 +518,11 @@ cudaError_t launch_energy_fp64(const Layout& L, const Precision& p, const void* 
     return dispatch_store(p.store, [&](auto tag) {
         using S = decltype(tag);
         const EnergyStrips es(L);
+        energy::Sum* const sums = reinterpret_cast<energy::Sum*>(part);   // 16 bytes a block
         auto* const kern = es.lw < 5 ? energy_kernel<S, true> : energy_kernel<S, false>;
         kern<<<nblk, kThreads, 0, st>>>(L, static_cast<const S*>(ang0), static_cast<const S*>(ang1), q,
-                                        fixed::turn_factor(q), es.rows, es.lw, part);
-        energy_final<<<1, kThreads, 0, st>>>(part, nblk, out);
+                                        fixed::turn_factor(q), es.rows, es.lw, sums);
+        energy_final<<<1, kThreads, 0, st>>>(sums, nblk, out);
         return cudaGetLastError();
     });
 }

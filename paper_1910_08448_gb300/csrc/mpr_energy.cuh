@@ -8,7 +8,7 @@
 // come by shuffle or are still in a register from the row above: 229 us at 4096^2 (one cosine per bond,
 // of the wrapped difference of the angles, 253 us; FP64 cosines 1625 us). A bond is off by at most 2^-55.6 (rms
 // 2^-57.5, mean 1.8e-18; q = 0.3, 0.5, 1 against 113 bits) and has 56 fraction bits. Sums are exact and do not depend on their order: 64-bit integers
-// within a strip, two FP64 words of whole numbers beyond; the only rounding is that of the result. (With
+// within a strip, two of them beyond; the only rounding is that of the result. (With
 // terms of 50 bits and sums of rounded FP64 strips the rms error of e_b was 1.1e-16 at 2 x 2, where
 // FP64 cosines give 4.5e-17; now 2.4e-17, and below FP64's at every size.)
 #pragma once
@@ -57,18 +57,39 @@ __device__ __forceinline__ int64_t term(Vec u, Vec h)
     return (e + 4) >> 2;
 }
 
-// A sum of terms as two FP64 words of whole numbers, 2^32 and 1 units of 2^-56: exact while they stay below
-// 2^53 (2^28 sites), beyond that good to 2^-53 of its size.
+// A bond energy in FP64 (an angle out of range) as a term; *nan is set for NaN.
+__device__ __forceinline__ int64_t term_fp64(double x, bool* nan)
+{
+    *nan |= isnan(x);
+    return __double2ll_rn(x * 0x1p56);
+}
+
+// A sum of terms, 2^32 and 1 units of 2^-56: exact. (FP64 words would be exact too, but the part adds 2 FP64 numbers
+// per SM and clock: 3 us longer at 100 x 70.)
 struct Sum {
-    double h, l;
+    long long h;
+    unsigned long long l;
     __device__ __forceinline__ void add(int64_t terms)
     {
-        h += (double)(int32_t)(terms >> 32);
-        l += (double)(uint32_t)terms;
+        h += terms >> 32;
+        l += (uint32_t)terms;
     }
-    __device__ __forceinline__ void add_fp64(double x) { l += x * 0x1p56; }
-    __device__ __forceinline__ double value() const { return h * 0x1p-24 + l * 0x1p-56; }
+    __device__ __forceinline__ void add(const Sum& o)
+    {
+        h += o.h;
+        l += o.l;
+    }
+    __device__ __forceinline__ void add_lane(int off)   // lane ^ off's
+    {
+        h += __shfl_xor_sync(0xffffffffu, h, off);
+        l += __shfl_xor_sync(0xffffffffu, l, off);
+    }
+    __device__ __forceinline__ double value() const
+    {
+        return (double)(h + (long long)(l >> 32)) * 0x1p-24 + (double)(uint32_t)l * 0x1p-56;
+    }
 };
+constexpr unsigned long long kNan = ~0ull;   // in place of l: the sum is NaN (l itself stays below 2^63)
 
 // Signed angles below 7.5 in size; other values (and NaN) are the caller's FP64 case.
 __device__ __forceinline__ bool in_range_signed(double x) { return fixed::in_range(fabs(x)); }
@@ -78,51 +99,41 @@ __device__ __forceinline__ uint64_t turns_signed(double x, fixed::Split k)
     return __double2hiint(x) < 0 ? 0ull - t : t;
 }
 
-// Sum over the block of one Sum per thread, in a fixed order (terms that were added in FP64), written by
-// thread 0 to the block's two words of part.
-__device__ __forceinline__ void block_sum(Sum v, double* part)
+// The sum over the block; valid in thread 0.
+__device__ __forceinline__ Sum block_sum(Sum v)
 {
     __shared__ Sum ws[kWarpsPerBlock];
 #pragma unroll
-    for (int off = 16; off; off >>= 1) {
-        v.h += __shfl_xor_sync(0xffffffffu, v.h, off);
-        v.l += __shfl_xor_sync(0xffffffffu, v.l, off);
-    }
+    for (int off = 16; off; off >>= 1) v.add_lane(off);
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        Sum s{0.0, 0.0};
-        for (int i = 0; i < kWarpsPerBlock; ++i) {
-            s.h += ws[i].h;
-            s.l += ws[i].l;
-        }
-        part[2 * blockIdx.x] = s.h;
-        part[2 * blockIdx.x + 1] = s.l;
-    }
+    if (threadIdx.x == 0)
+        for (int i = 1; i < kWarpsPerBlock; ++i) v.add(ws[i]);
+    return v;
 }
 
-// The sum of n blocks' words by one block, in a fixed order; valid in thread 0.
-__device__ __forceinline__ double final_sum(const double* __restrict__ part, int n)
+// The block's sum in its place of part; nan: a term of the thread is NaN.
+__device__ __forceinline__ void store_sum(Sum v, bool nan, Sum* part)
 {
-    __shared__ double sh[kThreads], sl[kThreads];
-    Sum s{0.0, 0.0};
+    const bool any = __syncthreads_or(nan);
+    v = block_sum(v);
+    if (any) v.l = kNan;
+    if (threadIdx.x == 0) part[blockIdx.x] = v;
+}
+
+// The sum of n blocks by one block; valid in thread 0.
+__device__ __forceinline__ double final_sum(const Sum* __restrict__ part, int n)
+{
+    Sum s{0, 0};
+    bool nan = false;
     for (int i = threadIdx.x; i < n; i += kThreads) {
-        s.h += part[2 * i];
-        s.l += part[2 * i + 1];
+        const Sum p = part[i];
+        nan |= p.l == kNan;
+        s.add(p);
     }
-    sh[threadIdx.x] = s.h;
-    sl[threadIdx.x] = s.l;
-    __syncthreads();
-    for (int w = kThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            sh[threadIdx.x] += sh[threadIdx.x + w];
-            sl[threadIdx.x] += sl[threadIdx.x + w];
-        }
-        __syncthreads();
-    }
-    s.h = sh[0];
-    s.l = sl[0];
-    return s.value();
+    const bool any = __syncthreads_or(nan);
+    s = block_sum(s);
+    return any ? (double)NAN : s.value();
 }
 
 }  // namespace energy

@@ -7,7 +7,7 @@
 // (reduction partials) inside a handle. This one keeps its scratch in a fixed array compiled into
 // the library instead, so a call only launches kernels.
 //
-// Cost of that choice: the array below (32 KiB of FP64 partials) exists on every GPU that loads
+// Cost of that choice: the array below (32 KiB of partial sums) exists on every GPU that loads
 // the library, for the life of the process, and all calls share it.
 #include "mpr.h"
 #include "mpr_energy.cuh"
@@ -24,13 +24,13 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr long long kMaxSites = 1ll << 28;    // 16384 x 16384
-constexpr int kPartials = 4096;               // words of the first pass's partial sums
+constexpr int kPartials = 2048;               // partial sums of the first pass, at most
 constexpr int kMaxDevices = 64;
 
-// The scratch: two words per block of the first pass (energy::Sum). Every block of a call writes its own
+// The scratch: one partial sum per block of the first pass (16 bytes). Every block of a call writes its own
 // slot before the second pass reads it, so nothing has to be cleared between calls. Calls that
 // overlap on the GPU (for example on two streams) use the same slots and race.
-static __device__ __align__(256) double g_bond_partials[kPartials];
+static __device__ __align__(256) mpr::energy::Sum g_bond_partials[kPartials];
 
 // First pass: sums of cos[q(phi_s - phi_right)] and cos[q(phi_s - phi_down)] (Eq. 2, open
 // boundaries). A strip is 31 columns x `rows` rows of one warp, lane 31 holding the right
@@ -39,7 +39,7 @@ static __device__ __align__(256) double g_bond_partials[kPartials];
 // 4096^2: 1612 us with two FP64 cosines per site on 256 blocks.
 __global__ void __launch_bounds__(kThreads) bond_partials(int Lx, int Ly, int rows,
                                                           const double* __restrict__ phi, double q,
-                                                          int64_t k65, double* __restrict__ part)
+                                                          int64_t k65, mpr::energy::Sum* __restrict__ part)
 {
     using namespace mpr;
     __shared__ fixed::Dir tab[fixed::kDirs];
@@ -49,7 +49,8 @@ __global__ void __launch_bounds__(kThreads) bond_partials(int Lx, int Ly, int ro
     const int lane = threadIdx.x & 31;
     const int nsx = (Lx + 30) / 31;
     const long long nstrips = (long long)nsx * ((Ly + rows - 1) / rows);
-    energy::Sum sum{0.0, 0.0};
+    energy::Sum sum{0, 0};
+    bool nan = false;
     for (long long st = (long long)blockIdx.x * energy::kWarpsPerBlock + (threadIdx.x >> 5);
          st < nstrips; st += (long long)gridDim.x * energy::kWarpsPerBlock) {
         const int sy = (int)(st / nsx), sx = (int)(st - (long long)sy * nsx);
@@ -74,8 +75,8 @@ __global__ void __launch_bounds__(kThreads) bond_partials(int Lx, int Ly, int ro
                 acc += mine ? e : 0;
             } else {
                 const double fr = __shfl_down_sync(0xffffffffu, f, 1);
-                if (right) sum.add_fp64(cos(q * (f - fr)));
-                if (mine && below) sum.add_fp64(cos(q * (f - fb)));
+                if (right) acc += energy::term_fp64(cos(q * (f - fr)), &nan);
+                if (mine && below) acc += energy::term_fp64(cos(q * (f - fb)), &nan);
             }
             f = fb;
             u = ub;
@@ -83,11 +84,11 @@ __global__ void __launch_bounds__(kThreads) bond_partials(int Lx, int Ly, int ro
         }
         sum.add(acc);
     }
-    energy::block_sum(sum, part);
+    energy::store_sum(sum, nan, part);
 }
 
 // Second pass, one block: fixed-order sum of the partials, e_b = -sum / N_b.
-__global__ void __launch_bounds__(kThreads) bond_final(const double* __restrict__ part, int nblk,
+__global__ void __launch_bounds__(kThreads) bond_final(const mpr::energy::Sum* __restrict__ part, int nblk,
                                                        double n_bonds, double* __restrict__ out)
 {
     const double s = mpr::energy::final_sum(part, nblk);
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(kThreads) bond_final(const double* __restrict_
 // for the life of the process. It belongs to the device's primary context: after a
 // cudaDeviceReset of that device the cached address is stale (see include/mpr.h).
 std::mutex g_mu;
-double* g_addr[kMaxDevices] = {};
+mpr::energy::Sum* g_addr[kMaxDevices] = {};
 
 mpr_status err(mpr_status s, const char* msg)
 {
@@ -127,7 +128,7 @@ extern "C" mpr_status mpr_bond_energy_noalloc(int Lx, int Ly, const double* angl
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
         return err(MPR_ERR_CUDA, "no usable current CUDA device");
-    double* part = nullptr;
+    mpr::energy::Sum* part = nullptr;
     {
         std::lock_guard<std::mutex> lock(g_mu);
         if (!g_addr[dev]) {
@@ -139,7 +140,7 @@ extern "C" mpr_status mpr_bond_energy_noalloc(int Lx, int Ly, const double* angl
                          cudaGetErrorString(e));
                 return err(MPR_ERR_CUDA, buf);
             }
-            g_addr[dev] = static_cast<double*>(p);
+            g_addr[dev] = static_cast<mpr::energy::Sum*>(p);
         }
         part = g_addr[dev];
     }
@@ -148,7 +149,7 @@ extern "C" mpr_status mpr_bond_energy_noalloc(int Lx, int Ly, const double* angl
     const int nsx = (Lx + 30) / 31, rows = mpr::energy::strip_rows(nsx, Ly);
     const long long strips = (long long)nsx * ((Ly + rows - 1) / rows);
     const int nblk = (int)std::min<long long>((strips + 7) / 8, 152 * 6);
-    static_assert(2 * 152 * 6 <= kPartials, "two words per block");
+    static_assert(152 * 6 <= kPartials, "one sum per block");
     const double n_bonds = (double)Lx * (Ly - 1) + (double)Ly * (Lx - 1);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     bond_partials<<<nblk, kThreads, 0, st>>>(Lx, Ly, rows, angles_dev, q,
