@@ -103,8 +103,8 @@ struct Split {
 
 MPR_HD constexpr Split split(int64_t a)
 {
-    // (the sum as unsigned: angles out of range pass here too, their result is not used)
-    return Split{(int32_t)((int64_t)((uint64_t)a + 0x80000000ull) >> 32), (int32_t)(uint32_t)a};
+    // h rounded to nearest (unsigned: angles out of range pass here too, their result is not used)
+    return Split{(int32_t)((uint32_t)(a >> 32) + ((uint32_t)a >> 31)), (int32_t)(uint32_t)a};
 }
 
 MPR_HD int32_t mulhi32(int32_t a, int32_t b) { return (int32_t)(((int64_t)a * b) >> 32); }
