@@ -186,6 +186,7 @@ KERNEL_SOURCES = {
     "mpr::sweep_f32_tma_kernel": ("mpr_tile_f32.cuh", "mpr_sweep_tma.cu", "mpr_tma.cuh",
                                   "mpr_device.cuh"),
     "mpr::sweep_kernel": ("mpr_sweep.cu", "mpr_fixed.cuh", "mpr_device.cuh"),
+    "mpr::resident": ("mpr_resident.cuh", "mpr_tile_f32.cuh", "mpr_device.cuh"),
 }
 
 
@@ -352,6 +353,8 @@ def run_mine(args, dist: Dist):
     mufu_peak = r_sc
     t_hbm = bytes_launch / (hbm_gbs * 1e9)
     kname = SWEEP_KERNELS[infos[-1]["sweep_kernel"]]
+    if infos[-1]["kernel_launches"] < infos[-1]["prof_sweep_launches"]:   # many passes in a launch
+        kname = "mpr::resident"
     kid = sweep_kernel_id(kname)
     workload = f"L{L}_p{p}_{args.setup}" + ("_bounded" if proposal else "")
     counters = stored_counters(kid, kname, workload)

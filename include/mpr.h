@@ -21,7 +21,10 @@
  *     pointers are device memory of the current CUDA device, e.g. from torch. The library copies
  *     inputs; the caller keeps ownership of every pointer it passes.
  *   - The library allocates the device memory of a handle at creation (from its stream-ordered
- *     pool, see mpr_trim_memory; batches with cudaMalloc) and frees it in mpr_destroy.
+ *     pool, see mpr_trim_memory; batches with cudaMalloc) and frees it in mpr_destroy. Runs and predictions
+ *     add what they first need: a word per measured sweep, a host prediction's staging (8 bytes per site), and
+ *     scratch of at most 20 MB and the boundary rows of resident sweeps, without which, when there is no memory
+ *     for it, runs go on more slowly.
  */
 #ifndef MPR_H
 #define MPR_H
@@ -43,7 +46,8 @@ typedef enum {
     MPR_ERR_TUNE_NO_CONVERGE = 4, /* sample energy above the bracket's top, or probes out   */
     MPR_ERR_CUDA = 5,             /* a CUDA runtime call failed                              */
     MPR_ERR_OOM = 6,              /* device allocation failed                                */
-    MPR_ERR_DEVICE_TIMEOUT = 7,   /* a bounded device-side wait ran out (batched kernel)    */
+    MPR_ERR_DEVICE_TIMEOUT = 7,   /* a bounded device-side wait ran out (TMA copy, rows of a
+                                     neighbouring band, grid barrier of a batch)            */
     MPR_ERR_STATE = 8             /* call out of order, e.g. predict before any sample       */
 } mpr_status;
 
@@ -98,9 +102,11 @@ typedef struct {
     size_t device_bytes;       /* device memory held by the handle                            */
     uint64_t kernel_launches;  /* kernels launched by the handle since creation               */
     double prof_sweep_ms;      /* with profiling on: device time of the pure sweep segments   */
-    uint64_t prof_sweep_launches; /* ... and the number of sweep-kernel launches they hold    */
-    int sweep_kernel;          /* FP32-function sweeps: 0 = one tile per block, 1 = TMA-fed   */
-                               /* persistent kernel; -1 = not chosen yet, or FP64 functions   */
+    uint64_t prof_sweep_launches; /* ... and the colour passes they hold, two per sweep: a launch  */
+                               /* each, or many in one launch where the sweeps run resident   */
+    int sweep_kernel;          /* FP32-function sweeps: 0 = one tile per block (or resident), */
+                               /* 1 = TMA-fed persistent kernel; -1 = not chosen yet, or FP64 */
+                               /* functions                                                   */
 } mpr_info;
 
 /* mpr_create: copies the host grid (values: Lx*Ly doubles, ignored where mask == 0 and may be
@@ -192,15 +198,22 @@ mpr_status mpr_get_info(mpr_handle h, mpr_info* info);
  * events on the handle's stream and accumulate their device time into prof_sweep_ms. */
 mpr_status mpr_set_profiling(mpr_handle h, int on);
 
-/* Sweep kernel of the FP32-function setups; both compute identical states, bit for bit.
+/* Sweep kernel of the FP32-function setups; all compute identical states, samples and energies, bit for bit.
  * kind 0: one tile (128 half-lattice columns x 32 rows) per block, staged with ordinary loads.
  * kind 1: persistent blocks over 128 x 32 tiles; the TMA unit copies the next tile's boxes into
  *         shared memory (cp.async.bulk.tensor, mbarrier with a bounded wait) while the block
  *         updates the current one. Needs a lattice at least two tiles wide (Lx > 256) and 34 rows.
- * kind -1 (default): automatic. The first run of at least 12 sweeps without energy or sample
- *         work (an equilibration, or a tuning probe's) times 5 sweeps of each kernel after one
- *         warm-up sweep each, as ordinary sweeps of the chain, and keeps kind 1 only if it is
- *         more than 2 % faster.
+ * kind -1 (default): automatic. Lattices up to about 1600 x 1600 run resident: uniform proposals, FP32 or 16-bit
+ *         spins, runs of two or more sweeps (three or four on some narrow grids). One launch runs up to 4096
+ *         sweeps; each block keeps a band of rows in shared memory and trades boundary rows with the blocks
+ *         beside it, in bounded waits. Such a launch keeps its SMs until its last sweep, so where several
+ *         handles or batches run on the device at the same time (calls in flight, counted by the library),
+ *         the larger of these lattices run one launch per colour pass instead, with kind 0; so does every
+ *         handle with kind 0 or 1 forced.
+ *         Elsewhere the first run of at least 12 sweeps without energy or sample work (an equilibration, or a
+ *         tuning probe's) times 5 sweeps of kinds 0 and 1 after one warm-up sweep each, as ordinary sweeps of the
+ *         chain, and keeps kind 1 only if it is more than 2 % faster. (A lattice that has run resident keeps
+ *         kind 0.)
  * INVALID_ARG if kind is not -1, 0 or 1, or kind 1 is unavailable for the handle. A forced kind
  * stays across mpr_set_options while it remains available; an automatic choice is redone. */
 mpr_status mpr_set_sweep_kernel(mpr_handle h, int kind);
@@ -252,9 +265,10 @@ mpr_status mpr_philox4x32_10_dev(const uint32_t* ctr_dev, uint32_t* out_dev, int
  * mask and temperature; problem i draws its random numbers from the Philox stream with problem id
  * i (so problem 0 of a batch follows the same chain as a single handle with the same options).
  * The batch computes with FP32 functions (opt->func must be MPR_PREC_S); storage, energy and
- * accumulator precision are free. The whole fill is ONE launch: by default a CUDA graph whose
- * device-side while loop repeats a red pass, a black pass (one block per tile of every unfinished
- * problem) and a finish kernel until every problem is done; or one persistent cooperative kernel
+ * accumulator precision are free. The whole fill is ONE launch: by default a CUDA graph with up to 8
+ * device-side while loops, side by side, one for each group of problems: a turn runs eight sweeps, a red and a
+ * black pass each (one block per tile of every unfinished problem), and a finish kernel, until every
+ * problem of the group is done; or one persistent cooperative kernel
  * whose blocks meet at grid barriers between colour passes. A barrier wait is bounded (2 s by
  * default) and a wait that runs out ends the launch with MPR_ERR_DEVICE_TIMEOUT (the batch is then
  * unusable).
@@ -273,11 +287,11 @@ mpr_status mpr_batch_set_tuning(mpr_batch b, const mpr_tuning* t);
  * 16 or 32 x 64 (64-column tiles waste less of narrow problems; default 32 x 128), blocks per SM
  * (persistent modes; 0 = occupancy limit) and mode: 0 = one persistent cooperative kernel (blocks
  * walk the tiles, grid barriers between colour passes), 1 = the same kernel as a one-node CUDA
- * graph, 2 (default) = one CUDA graph whose device-side while loop repeats a red pass, a black
- * pass (one block per tile) and a finish kernel until every problem is done. */
+ * graph, 2 (default) = one CUDA graph whose device-side while loops (one per group of problems) repeat eight
+ * sweeps, a red and a black pass each (one block per tile), and a finish kernel until every problem is done. */
 mpr_status mpr_batch_set_launch(mpr_batch b, int tile_rows, int tile_cols, int blocks_per_sm,
                                 int use_graph);
-/* Autotuner: times `sweeps` sweeps of every tile shape and mode (persistent modes at every
+/* Autotuner: times `sweeps` sweeps (rounded up to whole turns of eight) of every tile shape and mode (persistent modes at every
  * residency) on a copy of the batch state (the chains are left as they were), keeps the fastest,
  * and caches it for batches of the same signature. Any output pointer may be NULL. */
 mpr_status mpr_batch_autotune(mpr_batch b, int sweeps, int* tile_rows_out, int* tile_cols_out,

@@ -293,13 +293,13 @@ __global__ void __launch_bounds__(kThreads) energy_final(const energy::Sum* __re
 // Prediction zhat = zmin + (zmax - zmin) * (mean phi / 2*pi) on prediction sites, z elsewhere, as
 // zmin + sum * K with K = (zmax - zmin) / (2*pi*n) formed once per block: one FP64 multiply-add per
 // site (and one rounding less than dividing by n and by 2*pi at every site, which took about 20
-// instructions of the FP64 unit: 593 us at 4096^2, 9.4 ms at 16384^2). A block covers 256 columns
-// x kPredRows rows, all of a thread's loads in flight before K is ready; what is left is memory
-// traffic. On grids of at most 128 columns it covers 2^lw >= Lx columns and as many more rows, its rows
-// interleaved over the threads (2 x 1000000: 256 columns a block leave 254 of 256 threads idle).
-// Grids that would make fewer blocks than two per SM take one row per thread: there the FP64 unit's share
-// of a block is what the call waits for. With a range near the smallest FP64 numbers K would lose bits or vanish: 2^200 K then, and sums
-// times 2^-200 (both exact).
+// instructions of the FP64 unit: 593 us at 4096^2, 9.4 ms at 16384^2; now 71 us at 4096^2, at 65 % of
+// the DRAM rate, the FP64 unit 59 % busy). A block covers 256 columns x kPredRows rows, all of a thread's
+// loads in flight before K is ready. On grids of at most 128 columns it covers 2^lw >= Lx columns and as many
+// more rows, its rows interleaved over the threads (2 x 1000000: 256 columns a block leave 254 of 256
+// threads idle). Grids that would make fewer blocks than two per SM take one row per thread: there the
+// FP64 unit's share of a block is what the call waits for. With a range near the smallest FP64 numbers K
+// would lose bits or vanish: 2^200 K then, and sums times 2^-200 (both exact).
 // --------------------------------------------------------------------------------------------
 constexpr int kPredRows = 8;
 

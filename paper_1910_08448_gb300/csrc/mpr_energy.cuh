@@ -1,11 +1,11 @@
 // mpr_energy.cuh -- sums of bond energies cos[q(phi_i - phi_j)] (Eq. 2) in 64-bit fixed point
 // (mpr_fixed.cuh), for the energy of a state.
 //
-// What bounds them: instructions, 349 per site at 65 % of the issue slots (4096^2 counters; ALU 58 %, the
-// integer multiplies 31 % of the FMA pipes, DRAM 8 %). An FP64 cosine is about 20 instructions of a unit that
+// What bounds them: instructions, 315 per site at 64 % of the issue slots (4096^2 counters; ALU and the FMA pipe of
+// the integer multiplies 59 % each, DRAM 8 %). An FP64 cosine is about 20 instructions of a unit that
 // issues 2 per SM and clock. A warp walks down a strip of columns: each angle is loaded once and becomes a unit
 // vector once, a site's bonds are one product of its vector with the sum of its neighbours', which
-// come by shuffle or are still in a register from the row above: 229 us at 4096^2 (one cosine per bond,
+// come by shuffle or are still in a register from the row above: 213 us at 4096^2 (one cosine per bond,
 // of the wrapped difference of the angles, 253 us; FP64 cosines 1625 us). A bond is off by at most 2^-55.6 (rms
 // 2^-57.5, mean 1.8e-18; q = 0.3, 0.5, 1 against 113 bits) and has 56 fraction bits. Sums are exact and do not depend on their order: 64-bit integers
 // within a strip, two of them beyond; the only rounding is that of the result. (With

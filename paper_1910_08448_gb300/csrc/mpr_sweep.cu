@@ -17,8 +17,8 @@
 //     bound (about 1 in 10^4) is decided by the FP64 expression;
 //   - a local field below 2^-10, and a tile with an angle outside [0, 7.5) (a state set by the
 //     caller), take the FP64 functions throughout.
-// 4096^2, p = 0.9: 2889 -> 295 us per pass, 941 instructions per site at 68 % of the issue slots;
-// the half-rate integer multiplies (69 % of their pipe) come next. The rms error of a moved angle
+// 4096^2, p = 0.9: 2889 -> 266 us per pass, 860 instructions per site at 68 % of the issue slots; the ALU
+// (55 %) and the FMA pipe of the integer multiplies (53 %) come next. The rms error of a moved angle
 // against extended precision falls from 3.6e-16 ... 8.1e-16 to 1.5e-16 ... 2.4e-16 (q 0.3 ... 1).
 #include "mpr_device.cuh"
 #include "mpr_fixed.cuh"
