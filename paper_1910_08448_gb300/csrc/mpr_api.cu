@@ -605,10 +605,6 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
         if (!*ran) return MPR_OK;
         CU(cudaMemsetAsync(h->halo, 0, h->halo_bytes, h->stream));
     }
-    if (h->epoch > 0x7FFFFFFFu) {   // tags start again: no word of an earlier launch may carry one
-        if (h->halo) CU(cudaMemsetAsync(h->halo, 0, h->halo_bytes, h->stream));
-        h->epoch = 0;
-    }
     int most = std::min(n, kLongest);
     if (measure) {
         const size_t row = (size_t)h->L.Ly * p.G * 4, nt = (size_t)sweep_f32_blocks(h->L) * 8;
@@ -649,6 +645,10 @@ mpr_status resident_sweeps(mpr_ctx* h, int n, double T, int flags, bool* ran)
     for (int k = 0; k < n; k += m) {
         m = std::min(most, n - k);
         if (n - k - m == 1) --m;
+        if (h->epoch > 0x7FFFFFFFu) {   // tags start again: no word of an earlier launch may carry one
+            if (h->halo) CU(cudaMemsetAsync(h->halo, 0, h->halo_bytes, h->stream));
+            h->epoch = 0;
+        }
         a.nsweeps = m;
         a.sweep = h->sweep;
         a.depth = p.fine ? std::min(p.depth, 2 * (m - 1)) : 1;

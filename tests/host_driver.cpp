@@ -127,6 +127,42 @@ int main(int argc, char** argv)
         if (num(2) * num(3) <= 1400 * 1200 && !is_resident(fake::launches.front())) return 1;   // alone again
         for (mpr_handle g : others) mpr_destroy(g);
         mpr_destroy(h);
+    } else if (!strcmp(what, "tags")) {   // Lx Ly of a lattice on a grid: sweeps until the tags start again
+        // the first fields of resident::Args (mpr_resident.h)
+        struct Args {
+            int dims[8];
+            void* arrays[10];
+            float* er;
+            unsigned long long* halo;
+            uint32_t epoch;
+            int nsweeps;
+        };
+        mpr_handle h = handle(num(2), num(3));
+        uint64_t next = 0;   // tags up to here are taken
+        int restarts = 0;
+        bool ok = true;
+        fake::on_launch = [&](const fake::Launch& l) {
+            if (!is_resident(l)) return 0;
+            const Args& a = *static_cast<const Args*>(l.args[0]);
+            ok &= a.halo != nullptr && a.dims[0] == num(2) && a.dims[1] == num(3) && a.nsweeps >= 2;
+            if (a.epoch < next) {   // tags start again: no word of an earlier launch is left
+                ok &= a.epoch == 0 && *a.halo == 0;
+                ++restarts;
+            }
+            *a.halo = ~0ull;   // what a launch leaves
+            next = (uint64_t)a.epoch + 2ull * (uint64_t)a.nsweeps + 1;   // an exchange per pass, at most
+            ok &= next < (1ull << 32);
+            fake::launches.clear();
+            return 0;
+        };
+        const mpr_status s = mpr_run(h, 1500000000, 0);
+        fake::on_launch = nullptr;
+        report(s);
+        if (!ok || restarts != 1) {
+            fprintf(stderr, "ok %d, restarts %d\n", ok, restarts);
+            return 1;
+        }
+        mpr_destroy(h);
     } else if (!strcmp(what, "refuse")) {   // Lx Ly, error code of the resident launches
         mpr_handle h = handle(num(2), num(3));
         fake::launches.clear();

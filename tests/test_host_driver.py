@@ -141,3 +141,9 @@ def test_no_half_height_tiles_where_other_runs_fill_the_device(driver, shape, mo
         _, calls = driver("busy", *shape, others)
         plain = [a["grid"] for n, a in calls if _tile(n)][:10]
         assert len(plain) in (0, 10) and all((g > tiles) == (others + 1 <= most) for g in plain)
+
+
+# a grid's boundary rows carry tags that no earlier launch has used since the rows were last cleared
+@pytest.mark.parametrize("shape", [(300, 300), (777, 523)])
+def test_tags_start_again_with_cleared_rows(driver, shape):
+    assert driver("tags", *shape)[0] == 0
